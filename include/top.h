@@ -412,12 +412,11 @@ top_status top_coherence_intensity_backward(top_handle h, const top_grid* g, con
 
 /* Pass variants the autotuner chooses between, per line length M = P/2 (flags 0: the defaults).
  * Row passes of M (the x axis) read the row bits, the column pass of M (the y axis) the column
- * bit. TOP_TUNE_CLASSIC_*: the block-cooperative row kernels instead of the pair-local ones (plans
- * of one warp a half line at padding 2); TOP_TUNE_NO_L2_*: no L2 prefetch of the next wave's
- * inputs; bits 8-10 (TOP_TUNE_SPAN): fields per block of the inverse row pass with a field
- * epilogue, c -> 2^(c - 1) (0: 4); TOP_TUNE_THREE_PASS (read for M = 64): fields of 64 x 64 at
- * padding 2 go through the three passes and the workspace instead of the one-kernel on-chip
- * propagation (plain propagations: no modulation, a field epilogue). */
+ * bit. TOP_TUNE_NO_L2_*: no L2 prefetch of the next wave's inputs; TOP_TUNE_THREE_PASS (read for
+ * M = 64): fields of 64 x 64 at padding 2 go through the three passes and the workspace instead of
+ * the one-kernel on-chip propagation (plain propagations: no modulation, a field epilogue).
+ * TOP_TUNE_CLASSIC_* and TOP_TUNE_SPAN (bits 8-10, values 0 to 4) chose between row kernels that one
+ * kernel now replaces: still accepted, saved and loaded, without effect. */
 #define TOP_TUNE_CLASSIC_FWD 0x1u
 #define TOP_TUNE_CLASSIC_INV 0x2u
 #define TOP_TUNE_CLASSIC_CHAIN 0x4u

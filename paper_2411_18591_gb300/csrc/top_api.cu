@@ -251,6 +251,20 @@ float2 unit_root(long long m, long long n) {
 }
 
 // Stage twiddles w_{R SP}^{i j} of an engine plan, in the layout the device reads.
+std::vector<float2> twiddle_image(const EngineInfo& info) {
+  std::vector<float2> tw;
+  tw.reserve(info.tw_size);
+  int sp = info.M;
+  for (int s = 0; s < info.NS; ++s) {
+    const int r = info.R[s], L = sp;
+    sp /= r;
+    if (sp <= 1) continue;
+    for (int j = 1; j < r; ++j)
+      for (int i = 0; i < sp; ++i) tw.push_back(unit_root((long long)i * j, L));
+  }
+  return tw;
+}
+
 top_status engine_twiddles(top_handle h, int M, const float2** out) {
   auto it = h->eng_tw.find(M);
   if (it != h->eng_tw.end()) {
@@ -259,18 +273,8 @@ top_status engine_twiddles(top_handle h, int M, const float2** out) {
   }
   EngineInfo info;
   if (!find_engine(M, &info)) return fail(TOP_ERR_UNSUPPORTED, "no FFT engine for line length %d", M);
-  std::vector<float2> tw(std::max(1, info.tw_size));
-  size_t off = 0;
-  for (int s = 0; s < info.NS; ++s) {
-    int sp = 1;
-    for (int i = s + 1; i < info.NS; ++i) sp *= info.R[i];
-    if (sp <= 1) continue;
-    const int r = info.R[s], L = r * sp;
-    for (int j = 1; j < r; ++j)
-      for (int i = 0; i < sp; ++i) tw[off + size_t(j - 1) * sp + i] = unit_root((long long)i * j, L);
-    off += size_t(r - 1) * sp;
-  }
-  if ((int)off > std::max(1, info.tw_size)) return fail(TOP_ERR_INTERNAL, "twiddle table size mismatch");
+  const std::vector<float2> tw = twiddle_image(info);
+  if ((int)tw.size() != info.tw_size) return fail(TOP_ERR_INTERNAL, "twiddle table size mismatch");
   float2* d = nullptr;
   TOP_TRY(upload(h, tw, &d));
   h->eng_tw[M] = d;
@@ -279,19 +283,52 @@ top_status engine_twiddles(top_handle h, int M, const float2** out) {
 }
 
 // exp(-2 pi i p / P) for p < P / 2: the twiddles that fold and unfold the two halves.
+std::vector<float2> split_image(int P) {
+  std::vector<float2> w(P / 2);
+  for (int p = 0; p < P / 2; ++p) w[p] = unit_root(p, P);
+  return w;
+}
 top_status split_twiddles(top_handle h, int P, const float2** out) {
   auto it = h->split_tw.find(P);
   if (it != h->split_tw.end()) {
     *out = it->second;
     return TOP_OK;
   }
-  std::vector<float2> w(P / 2);
-  for (int p = 0; p < P / 2; ++p) w[p] = unit_root(p, P);
   float2* d = nullptr;
-  TOP_TRY(upload(h, w, &d));
+  TOP_TRY(upload(h, split_image(P), &d));
   h->split_tw[P] = d;
   *out = d;
   return TOP_OK;
+}
+
+// Geometry of a launch and the line order of its row plan.
+void set_geometry(PassParams& p, int ny, int nx, int Py, int Px) {
+  p.ny = ny;
+  p.nx = nx;
+  p.oy = (Py - ny) / 2;
+  p.ox = (Px - nx) / 2;
+  p.Py = Py;
+  p.Px = Px;
+  p.My = Py / 2;
+  p.Mx = Px / 2;
+  p.tune_rows = tune_flags(p.Mx);
+  p.tune_cols = tune_flags(p.My);
+  EngineInfo ex;
+  if (!find_engine(p.Mx, &ex)) return;
+  p.ci = ex.ci;
+  p.xstep = p.Mx / ex.R[ex.NS - 1];
+  p.xr0 = ex.NS == 3 ? ex.R[0] : 1;
+  p.xr1 = ex.NS == 3 ? ex.R[1] : 1;
+}
+
+// Quadrant table in the column plan's order (FieldSet::hq).
+cudaError_t build_transfer_table(float2* hq, int Py, int Px, double dy, double dx, double lam, double z, int method,
+                                 cudaStream_t s) {
+  EngineInfo ey;
+  if (!find_engine(Py / 2, &ey)) return cudaErrorInvalidValue;
+  const bool deep = ey.NS == 3;
+  return launch_transfer_table(hq, Py, Px, dy, dx, lam, z, method, ey.M / ey.R[ey.NS - 1], deep ? ey.R[0] : 1,
+                               deep ? ey.R[1] : 1, s);
 }
 
 long long signed_index(long long k, long long P) { return k < (P + 1) / 2 ? k : k - P; }
@@ -314,12 +351,7 @@ top_status di_table(top_handle h, int Py, int Px, double dy, double dx, double l
   float2* samples = static_cast<float2*>(buf);
   float2* ws = samples + plane;
   PassParams p{};
-  p.ny = Py;
-  p.nx = Px;
-  p.Py = Py;
-  p.Px = Px;
-  p.My = Py / 2;
-  p.Mx = Px / 2;
+  set_geometry(p, Py, Px, Py, Px);
   p.method = TOP_DI;
   p.src_kind = SRC_FIELD;
   p.epi_kind = EPI_FIELD;
@@ -368,7 +400,7 @@ top_status transfer_tables(top_handle h, int Py, int Px, double dy, double dx, d
   if (method == TOP_DI) {
     TOP_TRY(di_table(h, Py, Px, dy, dx, lam, z, st, te.hq));
   } else {
-    TOP_CUDA(launch_transfer_table(te.hq, Py, Px, dy, dx, lam, z, method, st), "transfer table");
+    TOP_CUDA(build_transfer_table(te.hq, Py, Px, dy, dx, lam, z, method, st), "transfer table");
   }
   TOP_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize(transfer table)");
   h->transfer[key] = te;
@@ -1044,27 +1076,8 @@ top_status run_bluestein(top_handle h, const Request& q, const Geometry& geo, cu
 
 top_status run_propagation(top_handle h, const Request& q, cudaStream_t st);
 
-// Whether every boundary of a request's upstream stages runs as one fused row pass: the next
-// stage's source operands fit the fused kernel's shared memory (as in run_chain).
-bool upstream_fuses(const Geometry& geo, const Request& q) {
-  EngineInfo ex;
-  if (!find_engine(geo.Px / 2, &ex)) return false;
-  for (int j = 0; j < q.n_up; ++j) {
-    PassParams probe{};
-    probe.nx = geo.nx;
-    probe.src_kind = SRC_FIELD;
-    probe.msrc = mod_dev(q.up[j].pre, 1, nullptr);
-    const size_t planes = src_plane_floats(probe, ex.rows);
-    const size_t rows_end = sizeof(float2) * (size_t(2) * ex.rows * ex.M + size_t(ex.rows) * geo.nx);
-    const size_t bytes = std::max(rows_end, ex.row_smem) + sizeof(float) * planes;
-    if (!((planes == 0 || geo.nx % 4 == 0) && bytes <= kChainSmemMax)) return false;
-  }
-  return true;
-}
-
 // The upstream stages of a request one propagation at a time through a field-sized scratch (sizes
-// without a plan of their own, or boundaries that do not fuse), then the request itself; the same
-// results as the fused passes.
+// without a plan of their own), then the request itself; the same results as the fused passes.
 top_status run_upstream_unfused(top_handle h, const Request& q, cudaStream_t st) {
   const int64_t B = q.g->batch;
   const size_t plane = size_t(q.g->ny) * size_t(q.g->nx);
@@ -1145,7 +1158,7 @@ top_status run_propagation(top_handle h, const Request& q, cudaStream_t st) {
       if (!std::isfinite(q.up[j].z)) return fail(TOP_ERR_INVALID_ARG, "stage %d: z must be finite", j);
       TOP_TRY(check_mod(q.up[j].pre, "stage modulation"));
     }
-    if (!planned || !upstream_fuses(geo, q)) return run_upstream_unfused(h, q, st);
+    if (!planned) return run_upstream_unfused(h, q, st);
   }
   if (!planned) return run_bluestein(h, q, geo, st);
   TOP_TRY(bind(h));
@@ -1284,16 +1297,7 @@ top_status run_propagation(top_handle h, const Request& q, cudaStream_t st) {
   }
 
   PassParams p{};
-  p.ny = geo.ny;
-  p.nx = geo.nx;
-  p.Py = geo.Py;
-  p.Px = geo.Px;
-  p.My = geo.Py / 2;
-  p.Mx = geo.Px / 2;
-  p.oy = geo.oy;
-  p.ox = geo.ox;
-  p.tune_rows = tune_flags(geo.Px / 2);
-  p.tune_cols = tune_flags(geo.Py / 2);
+  set_geometry(p, geo.ny, geo.nx, geo.Py, geo.Px);
   p.method = g->method;
   p.adjoint = q.adjoint;
   p.src_kind = q.src_kind;
@@ -1453,8 +1457,7 @@ top_status run_propagation(top_handle h, const Request& q, cudaStream_t st) {
 // ============================================================================= fused system chain
 
 // x_0 = in, x_k = P_{z_k}(pre_k x_{k-1}); the inverse row pass of stage k and the forward row
-// pass of stage k+1 run as one kernel where the next source's staged planes fit (else the pair
-// runs as two launches through `keep` or a field scratch in the workspace, with the same results).
+// pass of stage k+1 run as one kernel.
 top_status run_chain(top_handle h, const top_grid* g, const void* in, void* out, float* inten, int64_t group,
                      const double* lam, int64_t n_lz, const top_stage* stages, int K, cudaStream_t st) {
   Geometry geo;
@@ -1547,58 +1550,29 @@ top_status run_chain(top_handle h, const top_grid* g, const void* in, void* out,
   }
   auto same = [](const FieldSet& a, const FieldSet& b) { return std::memcmp(&a, &b, sizeof(FieldSet)) == 0; };
 
-  // stage boundaries that fuse: the next source's planes fit and are 16-byte rows
-  EngineInfo ex;
-  find_engine(geo.Px / 2, &ex);
-  std::vector<char> fused(K, 0);  // fused[k]: stage k-1 -> k in one kernel
-  bool scratch = false;
-  for (int k = 1; k < K; ++k) {
-    PassParams probe{};
-    probe.nx = geo.nx;
-    probe.src_kind = SRC_FIELD;
-    probe.msrc = mod_dev(stages[k].pre, 0, nullptr);
-    const size_t planes = src_plane_floats(probe, ex.rows);
-    // the field rows sit past the two half rows, the planes past the rows and the row-pass region
-    const size_t rows_end = sizeof(float2) * (size_t(2) * ex.rows * ex.M + size_t(ex.rows) * geo.nx);
-    const size_t bytes = std::max(rows_end, ex.row_smem) + sizeof(float) * planes;
-    fused[k] = (planes == 0 || geo.nx % 4 == 0) && bytes <= kChainSmemMax;
-    if (!fused[k] && !stages[k - 1].keep) scratch = true;
-  }
-
   const long long plane = (long long)geo.ny * geo.nx;
   const int64_t align = std::lcm(inten ? group : int64_t(1), in_repeat);
   if (align > kMaxFields) return fail(TOP_ERR_UNSUPPORTED, "intensity group larger than %d fields", kMaxFields);
   const size_t ws_field = size_t(geo.Px) * size_t(geo.ny) * sizeof(float2);
-  const size_t scr_field = scratch ? size_t(plane) * sizeof(float2) : 0;
   const bool share = in_repeat > 1 && shared_source(stages[0].pre);
   const size_t spec_src = share ? size_t(geo.Px) * size_t(geo.Py) * sizeof(float2) : 0;
   int64_t chunk = std::min<int64_t>(B, kMaxFields);
   chunk = std::max<int64_t>(align, chunk - chunk % align);
-  auto need = [&](int64_t c) { return size_t(c) * (ws_field + scr_field) + 256 + size_t(c / in_repeat) * spec_src + 256; };
+  auto need = [&](int64_t c) { return size_t(c) * ws_field + 256 + size_t(c / in_repeat) * spec_src + 256; };
   while (chunk > align && need(chunk) > h->ws_limit) chunk = std::max<int64_t>(align, (chunk / 2) - (chunk / 2) % align);
   if (need(chunk) > h->ws_limit)
     return fail(TOP_ERR_OOM, "one group of fields needs %zu bytes of workspace, above the limit %llu", need(chunk),
                 (unsigned long long)h->ws_limit);
   TOP_TRY(ensure_workspace(h, need(chunk)));
   float2* ws = static_cast<float2*>(h->ws);
-  float2* scr = scratch ? ws + size_t(chunk) * size_t(geo.Px) * size_t(geo.ny) : nullptr;
   float2* spec = nullptr;
   if (share) {
-    char* sb = reinterpret_cast<char*>(h->ws) + size_t(chunk) * (ws_field + scr_field);
+    char* sb = reinterpret_cast<char*>(h->ws) + size_t(chunk) * ws_field;
     spec = reinterpret_cast<float2*>((reinterpret_cast<uintptr_t>(sb) + 255) & ~uintptr_t(255));
   }
 
   PassParams base{};
-  base.ny = geo.ny;
-  base.nx = geo.nx;
-  base.Py = geo.Py;
-  base.Px = geo.Px;
-  base.My = geo.Py / 2;
-  base.Mx = geo.Px / 2;
-  base.oy = geo.oy;
-  base.ox = geo.ox;
-  base.tune_rows = tune_flags(geo.Px / 2);
-  base.tune_cols = tune_flags(geo.Py / 2);
+  set_geometry(base, geo.ny, geo.nx, geo.Py, geo.Px);
   base.method = g->method;
   base.src_kind = SRC_FIELD;
   base.epi_kind = EPI_FIELD;
@@ -1681,17 +1655,8 @@ top_status run_chain(top_handle h, const top_grid* g, const void* in, void* out,
       TOP_TRY(timed(h, KK_COLS, st, "column pass", [&] { return launch_pass(PASS_COLS, geo.Py / 2, ps[0], st); }));
     }
     for (int k = 1; k < K; ++k) {
-      if (fused[k]) {
-        TOP_TRY(timed(h, KK_ROWS_CHAIN, st, "fused row pass",
-                      [&] { return launch_pass(PASS_ROWS_CHAIN, geo.Px / 2, ps[k - 1], st, &ps[k]); }));
-      } else {
-        // two launches through the kept field or the scratch
-        PassParams pa = ps[k - 1], pb = ps[k];
-        if (!pa.out) pa.out = scr;
-        pb.in = pa.out;
-        TOP_TRY(timed(h, KK_ROWS_INV, st, "rows inverse pass", [&] { return launch_pass(PASS_ROWS_INV, geo.Px / 2, pa, st); }));
-        TOP_TRY(timed(h, KK_ROWS_FWD, st, "rows forward pass", [&] { return launch_pass(PASS_ROWS_FWD, geo.Px / 2, pb, st); }));
-      }
+      TOP_TRY(timed(h, KK_ROWS_CHAIN, st, "fused row pass",
+                    [&] { return launch_pass(PASS_ROWS_CHAIN, geo.Px / 2, ps[k - 1], st, &ps[k]); }));
       TOP_TRY(timed(h, KK_COLS, st, "column pass", [&] { return launch_pass(PASS_COLS, geo.Py / 2, ps[k], st); }));
     }
     TOP_TRY(timed(h, KK_ROWS_INV, st, "rows inverse pass", [&] { return launch_pass(PASS_ROWS_INV, geo.Px / 2, last, st); }));
@@ -1778,16 +1743,7 @@ top_status run_ragged(top_handle h, int count, const top_grid* grids, const void
     void** d_lists = reinterpret_cast<void**>(tail);  // [in][out][table], chunk entries each
 
     PassParams p{};
-    p.ny = geo.ny;
-    p.nx = geo.nx;
-    p.Py = geo.Py;
-    p.Px = geo.Px;
-    p.My = geo.Py / 2;
-    p.Mx = geo.Px / 2;
-    p.oy = geo.oy;
-    p.ox = geo.ox;
-    p.tune_rows = tune_flags(geo.Px / 2);
-    p.tune_cols = tune_flags(geo.Py / 2);
+    set_geometry(p, geo.ny, geo.nx, geo.Py, geo.Px);
     p.method = grids[grp[0]].method;
     p.adjoint = backward ? 1 : 0;
     p.src_kind = SRC_FIELD;
@@ -1955,12 +1911,9 @@ top_status top_autotune(top_handle h, const top_grid* g, uint32_t* rows_flags, u
     h->pending.clear();
     return TOP_OK;
   };
-  double A[KK_COUNT], Bc[KK_COUNT], C[KK_COUNT], D[KK_COUNT], E[KK_COUNT];
+  double A[KK_COUNT], C[KK_COUNT];
   top_status st = measure(0, 0, A);
-  if (st == TOP_OK) st = measure(TOP_TUNE_CLASSIC_FWD | TOP_TUNE_CLASSIC_INV | TOP_TUNE_CLASSIC_CHAIN, 0, Bc);
-  if (st == TOP_OK) st = measure(TOP_TUNE_NO_L2_FWD | TOP_TUNE_SPAN(1), TOP_TUNE_NO_L2_COLS, C);
-  if (st == TOP_OK) st = measure(TOP_TUNE_SPAN(2), 0, D);
-  if (st == TOP_OK) st = measure(TOP_TUNE_SPAN(4), 0, E);
+  if (st == TOP_OK) st = measure(TOP_TUNE_NO_L2_FWD, TOP_TUNE_NO_L2_COLS, C);
   h->prof = keep_prof;
   cudaFree(x);
   cudaFree(y);
@@ -1972,19 +1925,8 @@ top_status top_autotune(top_handle h, const top_grid* g, uint32_t* rows_flags, u
   }
   // a variant replaces the default only when it is more than 2 % faster
   auto better = [](double cand, double base) { return cand < 0.98 * base; };
-  uint32_t rows = 0, cols = 0;
-  double fwd = A[KK_ROWS_FWD];
-  if (better(Bc[KK_ROWS_FWD], fwd)) { rows |= TOP_TUNE_CLASSIC_FWD; fwd = Bc[KK_ROWS_FWD]; }
-  if (better(C[KK_ROWS_FWD], fwd)) { rows = (rows & ~TOP_TUNE_CLASSIC_FWD) | TOP_TUNE_NO_L2_FWD; }
-  double inv = A[KK_ROWS_INV];
-  uint32_t inv_bits = 0;
-  const std::pair<double, uint32_t> inv_cands[] = {{Bc[KK_ROWS_INV], TOP_TUNE_CLASSIC_INV}, {C[KK_ROWS_INV], TOP_TUNE_SPAN(1)},
-                                                   {D[KK_ROWS_INV], TOP_TUNE_SPAN(2)}, {E[KK_ROWS_INV], TOP_TUNE_SPAN(4)}};
-  for (const auto& c : inv_cands)
-    if (better(c.first, inv)) { inv = c.first; inv_bits = c.second; }
-  rows |= inv_bits;
-  if (better(Bc[KK_ROWS_CHAIN], A[KK_ROWS_CHAIN])) rows |= TOP_TUNE_CLASSIC_CHAIN;
-  if (better(C[KK_COLS], A[KK_COLS])) cols |= TOP_TUNE_NO_L2_COLS;
+  const uint32_t rows = better(C[KK_ROWS_FWD], A[KK_ROWS_FWD]) ? TOP_TUNE_NO_L2_FWD : 0;
+  const uint32_t cols = better(C[KK_COLS], A[KK_COLS]) ? TOP_TUNE_NO_L2_COLS : 0;
   apply(rows, cols);
   if (rows_flags) *rows_flags = tune_flags(Mx);
   if (cols_flags) *cols_flags = tune_flags(My);
@@ -2708,23 +2650,6 @@ top_status noalloc_scratch(void** out) {
   return TOP_OK;
 }
 
-// Host image of an engine's stage twiddles (the same float64 arithmetic as the handle's cached ones).
-void noalloc_engine_twiddles(int M, std::vector<float2>& tw) {
-  EngineInfo info;
-  find_engine(M, &info);
-  tw.assign(std::max(1, info.tw_size), make_float2(0.f, 0.f));
-  size_t off = 0;
-  for (int s = 0; s < info.NS; ++s) {
-    int sp = 1;
-    for (int i = s + 1; i < info.NS; ++i) sp *= info.R[i];
-    if (sp <= 1) continue;
-    const int r = info.R[s], L = r * sp;
-    for (int j = 1; j < r; ++j)
-      for (int i = 0; i < sp; ++i) tw[off + size_t(j - 1) * sp + i] = unit_root((long long)i * j, L);
-    off += size_t(r - 1) * sp;
-  }
-}
-
 // Append a table to the host image at a 256-byte boundary; returns its byte offset.
 template <class T>
 size_t put(std::vector<unsigned char>& img, const std::vector<T>& v) {
@@ -2752,8 +2677,7 @@ top_status propagate_noalloc(const top_grid* g, const void* in, void* out, const
   EngineInfo ix, iy;
   find_engine(geo.Px / 2, &ix);
   find_engine(geo.Py / 2, &iy);
-  const size_t tw_bytes = align256(std::max(1, ix.tw_size) * sizeof(float2)) +
-                          align256(std::max(1, iy.tw_size) * sizeof(float2)) +
+  const size_t tw_bytes = align256(ix.tw_size * sizeof(float2)) + align256(iy.tw_size * sizeof(float2)) +
                           align256(size_t(geo.Px / 2) * sizeof(float2)) + align256(size_t(geo.Py / 2) * sizeof(float2));
   const size_t set_bytes = align256(size_t(geo.Px / 2 + 1) * size_t(geo.Py / 2 + 2) * sizeof(float2));
   const size_t ws_field = size_t(geo.Px) * size_t(geo.ny) * sizeof(float2);
@@ -2787,28 +2711,15 @@ top_status propagate_noalloc(const top_grid* g, const void* in, void* out, const
 
   // twiddles: written in stream order by kernels that carry them in their parameters (no copy from
   // pageable host memory)
-  std::vector<float2> twx, twy, wpx(geo.Px / 2), wpy(geo.Py / 2);
-  noalloc_engine_twiddles(geo.Px / 2, twx);
-  noalloc_engine_twiddles(geo.Py / 2, twy);
-  for (int q = 0; q < geo.Px / 2; ++q) wpx[q] = unit_root(q, geo.Px);
-  for (int q = 0; q < geo.Py / 2; ++q) wpy[q] = unit_root(q, geo.Py);
   std::vector<unsigned char> img;
-  const size_t o_twx = put(img, twx), o_twy = put(img, twy), o_wpx = put(img, wpx), o_wpy = put(img, wpy);
+  const size_t o_twx = put(img, twiddle_image(ix)), o_twy = put(img, twiddle_image(iy));
+  const size_t o_wpx = put(img, split_image(geo.Px)), o_wpy = put(img, split_image(geo.Py));
   if (img.size() > tw_bytes) return fail(TOP_ERR_INTERNAL, "static twiddle image above its reserved size");
   img.resize((img.size() + 7) & ~size_t(7));
   TOP_CUDA(launch_put(base, img.data(), img.size(), st), "static twiddles");
 
   PassParams p{};
-  p.ny = geo.ny;
-  p.nx = geo.nx;
-  p.Py = geo.Py;
-  p.Px = geo.Px;
-  p.My = geo.Py / 2;
-  p.Mx = geo.Px / 2;
-  p.oy = geo.oy;
-  p.ox = geo.ox;
-  p.tune_rows = tune_flags(geo.Px / 2);
-  p.tune_cols = tune_flags(geo.Py / 2);
+  set_geometry(p, geo.ny, geo.nx, geo.Py, geo.Px);
   p.method = g->method;
   p.adjoint = 0;
   p.src_kind = SRC_FIELD;
@@ -2845,7 +2756,7 @@ top_status propagate_noalloc(const top_grid* g, const void* in, void* out, const
         if ((int)keys.size() == slots) break;
         keys.push_back(key);
         float2* hq = reinterpret_cast<float2*>(base + tw_bytes + k * set_bytes);
-        TOP_CUDA(launch_transfer_table(hq, geo.Py, geo.Px, g->dy, g->dx, lam[i], z[i], g->method, st), "transfer table");
+        TOP_CUDA(build_transfer_table(hq, geo.Py, geo.Px, g->dy, g->dx, lam[i], z[i], g->method, st), "transfer table");
         FieldSet fs{};
         fs.hq = hq;
         p.sets[k] = fs;

@@ -195,7 +195,7 @@ __device__ __forceinline__ float2 transfer_value(int akx, int aky, int Py, int P
 }
 
 __global__ void __launch_bounds__(256) k_transfer_table(float2* hq, int Py, int Px, double dy, double dx, double lam,
-                                                        double z, int method) {
+                                                        double z, int method, int S, int r0, int r1) {
   const int my = Py / 2, even = my / 2 + 1;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   const int akx = blockIdx.y;
@@ -205,7 +205,10 @@ __global__ void __launch_bounds__(256) k_transfer_table(float2* hq, int Py, int 
     *out = make_float2(0.f, 0.f);
     return;
   }
-  const int aky = j < even ? 2 * j : 2 * (j - even) + 1;
+  const int e = j < even ? j : j - even;  // entry of the part
+  const int b = e % S;
+  const int k = b / r1 + (b % r1) * r0 + (e - b);
+  const int aky = j < even ? 2 * k : 2 * k + 1;
   *out = transfer_value(akx, aky, Py, Px, dy, dx, lam, z, method);
 }
 
@@ -552,10 +555,10 @@ cudaError_t launch_resample(const float2* in, float2* out, long long batch, Resa
 }
 
 cudaError_t launch_transfer_table(float2* hq, int Py, int Px, double dy, double dx, double lam, double z, int method,
-                                  cudaStream_t s) {
+                                  int S, int r0, int r1, cudaStream_t s) {
   const int my = Py / 2;
   dim3 grid((my + 2 + 255) / 256, Px / 2 + 1);
-  TOP_LAUNCH(k_transfer_table, grid, 256, 0, s, hq, Py, Px, dy, dx, lam, z, method);
+  TOP_LAUNCH(k_transfer_table, grid, 256, 0, s, hq, Py, Px, dy, dx, lam, z, method, S, r0, r1);
   return cudaGetLastError();
 }
 

@@ -60,9 +60,10 @@ struct ResampleGeom {
 };
 cudaError_t launch_resample(const float2* in, float2* out, long long batch, ResampleGeom rg, int transpose,
                             cudaStream_t s);
-// Quadrant table of H / (Py Px) for one (lambda, z) in the FieldSet::hq layout (float64 arithmetic).
+// Quadrant table of H / (Py Px) for one (lambda, z) in the FieldSet::hq layout (float64 arithmetic);
+// the column plan's order: entry b + S j of a part holds k = b / r1 + (b % r1) r0 + S j.
 cudaError_t launch_transfer_table(float2* hq, int Py, int Px, double dy, double dx, double lam, double z, int method,
-                                  cudaStream_t s);
+                                  int S, int r0, int r1, cudaStream_t s);
 // The same values on the whole grid in natural order, h[kx Py + ky] (the Bluestein column lines).
 cudaError_t launch_transfer_full(float2* h, int Py, int Px, double dy, double dx, double lam, double z, int method,
                                  cudaStream_t s);

@@ -15,7 +15,7 @@ struct EngineInfo {
   int R[4];   // radices
   int tw_size;
   int rows;         // rows per block of the row passes
-  size_t row_smem;  // shared memory of a row block before any staged planes
+  int ci;           // workspace lines interleaved by the row passes
 };
 
 // PASS_ROWS_CHAIN: the inverse row pass of one propagation fused with the forward row pass of

@@ -48,8 +48,8 @@ __device__ __forceinline__ float2 c_sub(float2 a, float2 b) {
 }
 // Scalar forms, where an operand is a quarter-turn rotation that the scalar instructions absorb
 // (a packed pair would need the swapped components moved into a register pair first).
-__device__ __forceinline__ float2 s_add(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 s_sub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 s_add(float2 a, float2 b) { return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y)); }
+__device__ __forceinline__ float2 s_sub(float2 a, float2 b) { return make_float2(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y)); }
 __device__ __forceinline__ float2 c_mul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -168,10 +168,9 @@ __device__ __forceinline__ void dft3(float2* v) {
   const float2 x0 = v[0], x1 = v[S], x2 = v[2 * S];
   const float2 t = c_add(x1, x2), d = c_sub(x1, x2);
   const float2 m = make_float2(fmaf(c, t.x, x0.x), fmaf(c, t.y, x0.y));
-  const float2 id = make_float2(-s * d.y, s * d.x);  // i s d
   v[0] = c_add(x0, t);
-  v[S] = s_add(m, id);
-  v[2 * S] = s_sub(m, id);
+  v[S] = make_float2(fmaf(-s, d.y, m.x), fmaf(s, d.x, m.y));  // m + i s d
+  v[2 * S] = make_float2(fmaf(s, d.y, m.x), fmaf(-s, d.x, m.y));
 }
 
 template <int S, int DIR>
@@ -296,27 +295,32 @@ struct Engine : Radices<R0, R1, R2, R3> {
   static constexpr int M = M_;
   static constexpr int G = G_;
   static constexpr int E = M / G;
+  // Threads a line group takes in a block: G where groups tile a warp, else the next whole number
+  // of warps. The spare threads of a padded group repeat its last lane's work on the same addresses
+  // (same values in the same instruction), so every group synchronises without the rest of the block.
+  static constexpr int GW = (G <= 32 && 32 % G == 0) ? G : ((G + 31) / 32) * 32;
   static_assert(R0 * R1 * R2 * R3 == M, "radices must multiply to M");
   static_assert(M % G == 0, "G must divide M");
   static_assert(Rd::divides(M_, G_), "G must divide M / R_s for every stage");
   static constexpr int TW_SIZE = Rd::tw_off(Rd::NS) > 0 ? Rd::tw_off(Rd::NS) : 1;
-  static constexpr int PADW = M / 4 >= 32 ? 32 : (M / 4 >= 1 ? M / 4 : 1);
-  // padded line buffer (float2 elements) with one spare slot between lines
-  static constexpr int BUF = (M - 1) + (M - 1) / PADW + 2;
   static constexpr int RL = Rd::radix(Rd::NS - 1);
+  // Padded line buffer (float2 elements): one spare slot per PADW samples, chosen per plan by
+  // simulating the banks for the exchanges' writes and reads (two wavefronts per 8-byte warp access,
+  // the minimum, for the power-of-two plans; up to 3 for the plans with factors of 5).
+  static constexpr int PADW = M % 5 == 0 ? 4 : (RL == 32 || M >= 2048) ? 32 : M >= 128 ? 16 : (M >= 64 ? 8 : M / 4);
+  static constexpr int BUF = (M - 1) + (M - 1) / PADW + 2;
+  static constexpr int SL = M / RL;  // bins between consecutive outputs of a last-stage butterfly
 
   __device__ __forceinline__ static int padi(int p) { return p + p / PADW; }
 
   // a group that tiles a warp synchronises with __syncwarp, a group of whole warps with its own
   // named barrier (ids from 15 down, one per group of the block; the pass shapes assert that they
-  // stay clear of the column barriers' ids from 1 up), anything else with the whole block
+  // stay clear of the other barriers' ids from 1 up)
   __device__ __forceinline__ static void sync_group() {
-    if constexpr (G <= 32 && 32 % G == 0) {
+    if constexpr (GW <= 32) {
       __syncwarp();
-    } else if constexpr (G % 32 == 0) {
-      top_named_barrier(15 - int(threadIdx.x) / G, G);
     } else {
-      __syncthreads();
+      top_named_barrier(15 - int(threadIdx.x) / GW, GW);
     }
   }
 
@@ -346,15 +350,17 @@ struct Engine : Radices<R0, R1, R2, R3> {
     }
     return k;
   }
+  // the butterfly index b with kbase(b) == m (0 <= m < SL)
+  __host__ __device__ __forceinline__ static constexpr int kbase_inv(int m) {
+    int b = 0;
+#pragma unroll
+    for (int s = 0; s < NS - 1; ++s) b += ((m / weight(s)) % radix(s)) * (span(s) / RL);
+    return b;
+  }
   __device__ __forceinline__ static int bin(int t, int e) {
     const int q = e / RL, j = e - (e / RL) * RL;
     return kbase(t + G * q) + j * (M / RL);
   }
-  // Arrays indexed by bin that lanes read or write in the frequency layout: where consecutive
-  // lanes hold bins a multiple of 16 apart (sixteen 8-byte entries span the banks once), one
-  // spare entry after every 16 spreads a warp's accesses over all banks.
-  static constexpr bool BIN_PAD = (kbase(1) - kbase(0)) % 16 == 0;
-  __host__ __device__ __forceinline__ static constexpr int bin_slot(int k) { return BIN_PAD ? k + k / 16 : k; }
 
   template <int S, int DIR>
   __device__ __forceinline__ static void stage(float2 (&v)[E], int t, const float2* __restrict__ tw) {
@@ -382,72 +388,120 @@ struct Engine : Radices<R0, R1, R2, R3> {
     }
   }
 
+  template <int A>
+  __device__ __forceinline__ static void put(const float2 (&v)[E], float2* __restrict__ buf, int t) {
+    constexpr int R = radix(A), Q = M / (R * G);
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+#pragma unroll
+      for (int j = 0; j < R; ++j) buf[padi(pos<A>(t, q, j))] = v[q * R + j];
+  }
+  template <int A>
+  __device__ __forceinline__ static void get(float2 (&v)[E], const float2* __restrict__ buf, int t) {
+    constexpr int R = radix(A), Q = M / (R * G);
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+#pragma unroll
+      for (int j = 0; j < R; ++j) v[q * R + j] = buf[padi(pos<A>(t, q, j))];
+  }
   template <int A, int B>
   __device__ __forceinline__ static void exchange(float2 (&v)[E], float2* __restrict__ buf, int t) {
-    constexpr int RA = radix(A), QA = M / (RA * G);
-    constexpr int RB = radix(B), QB = M / (RB * G);
     sync_group();
-#pragma unroll
-    for (int q = 0; q < QA; ++q)
-#pragma unroll
-      for (int j = 0; j < RA; ++j) buf[padi(pos<A>(t, q, j))] = v[q * RA + j];
+    put<A>(v, buf, t);
     sync_group();
-#pragma unroll
-    for (int q = 0; q < QB; ++q)
-#pragma unroll
-      for (int j = 0; j < RB; ++j) v[q * RB + j] = buf[padi(pos<B>(t, q, j))];
+    get<B>(v, buf, t);
   }
-
-  // fwd_compact / inv_compact: two-stage plans with equal radices run their two stages as one loop
-  // over a single copy of the in-register DFT (half the code of the unrolled form), for kernels
-  // whose code otherwise spills out of the instruction cache (the fused row passes hold a forward
-  // and an inverse transform); elsewhere the unrolled form measured faster.
-  static constexpr bool LOOP2 = NS == 2 && Rd::radix(0) == Rd::radix(1);
 
   template <int DIR>
   __device__ __forceinline__ static void dfts(float2 (&v)[E]) {
-    constexpr int R = radix(0), Q = M / (R * G);
 #pragma unroll
-    for (int q = 0; q < Q; ++q) dft<R, 1, DIR>(v + q * R);
+    for (int q = 0; q < E / R0; ++q) dft<R0, 1, DIR>(v + q * R0);
   }
   // the twiddles of stage 0 (span span(0)), conjugated for the inverse
   template <int DIR>
   __device__ __forceinline__ static void stage0_twiddles(float2 (&v)[E], int t, const float2* __restrict__ tw) {
-    constexpr int R = radix(0), SP = span(0), Q = M / (R * G);
+    constexpr int SP = span(0);
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      float2* w = v + q * R;
-      const int i = (t + G * q) % SP;
-      const float2* tp = tw + tw_off(0) + i;
+    for (int q = 0; q < E / R0; ++q) {
+      float2* w = v + q * R0;
+      const float2* tp = tw + t + G * q;
 #pragma unroll
-      for (int j = 1; j < R; ++j) w[j] = DIR < 0 ? c_mul(w[j], __ldg(tp + (j - 1) * SP)) : c_mulc(w[j], __ldg(tp + (j - 1) * SP));
+      for (int j = 1; j < R0; ++j) w[j] = DIR < 0 ? c_mul(w[j], __ldg(tp + (j - 1) * SP)) : c_mulc(w[j], __ldg(tp + (j - 1) * SP));
     }
   }
 
-  __device__ __forceinline__ static void fwd_compact(float2 (&v)[E], float2* buf, int t, const float2* __restrict__ tw) {
-    if constexpr (LOOP2) {
+  // COMPACT runs the two stages of a plan with equal radices as one loop over a single copy of the
+  // in-register DFT (half the code), for kernels whose code otherwise spills out of the instruction
+  // cache; elsewhere the unrolled form measured faster.
+  static constexpr bool LOOP2 = NS == 2 && Rd::radix(0) == Rd::radix(1);
+
+  // Forward transform whose last exchange may hand the line to other threads: this thread writes as
+  // lane t of the line at `buf` and, after `read_ready`, reads as lane rt of the line at `rbuf`.
+  // `buf_free` runs before the first write to `buf`.
+  template <bool COMPACT, class SF, class SR>
+  __device__ __forceinline__ static void fwd_to(float2 (&v)[E], float2* buf, int t, const float2* __restrict__ tw,
+                                                SF&& buf_free, const float2* rbuf, int rt, SR&& read_ready) {
+    if constexpr (COMPACT && LOOP2) {
 #pragma unroll 1
       for (int s = 0; s < 2; ++s) {
-        if (s == 1) exchange<0, 1>(v, buf, t);
+        if (s == 1) {
+          buf_free();
+          put<0>(v, buf, t);
+          read_ready();
+          get<1>(v, rbuf, rt);
+        }
         dfts<-1>(v);
         if (s == 0) stage0_twiddles<-1>(v, t, tw);
       }
     } else {
-      fwd(v, buf, t, tw);
+      stage<0, -1>(v, t, tw);
+      buf_free();
+      put<0>(v, buf, t);
+      if constexpr (NS == 3) {
+        sync_group();
+        get<1>(v, buf, t);
+        stage<1, -1>(v, t, tw);
+        sync_group();
+        put<1>(v, buf, t);
+      }
+      static_assert(NS == 2 || NS == 3, "two or three stages");
+      read_ready();
+      get<NS - 1>(v, rbuf, rt);
+      stage<NS - 1, -1>(v, rt, tw);
     }
   }
-  __device__ __forceinline__ static void inv_compact(float2 (&v)[E], float2* buf, int t, const float2* __restrict__ tw) {
-    if constexpr (LOOP2) {
+
+  // The inverse of fwd_to, unnormalised: bins held as lane rt of the line at rbuf, to natural order as
+  // lane t of the line at buf.
+  template <bool COMPACT, class SF, class SR>
+  __device__ __forceinline__ static void inv_from(float2 (&v)[E], float2* rbuf, int rt, SF&& buf_free, float2* buf, int t,
+                                                  SR&& read_ready, const float2* __restrict__ tw) {
+    if constexpr (COMPACT && LOOP2) {
 #pragma unroll 1
       for (int s = 0; s < 2; ++s) {
         if (s == 1) {
-          exchange<1, 0>(v, buf, t);
+          buf_free();
+          put<1>(v, rbuf, rt);
+          read_ready();
+          get<0>(v, buf, t);
           stage0_twiddles<+1>(v, t, tw);
         }
         dfts<+1>(v);
       }
     } else {
-      inv(v, buf, t, tw);
+      stage<NS - 1, +1>(v, rt, tw);
+      buf_free();
+      put<NS - 1>(v, rbuf, rt);
+      read_ready();
+      if constexpr (NS == 3) {
+        get<1>(v, buf, t);
+        stage<1, +1>(v, t, tw);
+        sync_group();
+        put<1>(v, buf, t);
+        sync_group();
+      }
+      get<0>(v, buf, t);
+      stage<0, +1>(v, t, tw);
     }
   }
 

@@ -20,9 +20,10 @@ constexpr int kMaxFields = 2048;  // fields per launch (larger batches run in ch
 // One (lambda, z) parameter set: the transfer function and the lens factors, computed in
 // float64 and rounded to float32. H depends on the frequencies only through fx^2 and fy^2, so
 // one quadrant is stored: hq[|kx| (My + 2) + j] = H(|kx|, |ky|) / (Py Px) for |kx| <= Px / 2,
-// with the even |ky| = 2 j at j < My/2 + 1, the odd |ky| = 2 (j - My/2 - 1) + 1 after them and
-// one zero entry that makes rows whole 16-byte units (one row per |kx|; a column half reads the
-// even or the odd part of its row).
+// with the even |ky| = 2 k (k <= My/2) in the first My/2 + 1 entries, the odd |ky| = 2 k + 1
+// (k < My/2) after them and one zero entry (one row per |kx|; a column half reads the even or the
+// odd part of its row). Within a part, k sits where the column plan's lanes hold the bin: k =
+// kbase(b) + S j at b + S j (S = My / RL; the identity for two-stage plans).
 struct FieldSet {
   const float2* hq;      // [Px/2 + 1][My + 2]
   const float2* src_lx;  // lens factor tables of the source-side modulation: [nx], [ny]
@@ -60,6 +61,8 @@ struct PassParams {
   int Py, Px;      // padded sizes (even; each handled as two interleaved halves)
   int My, Mx;      // Py / 2, Px / 2
   int oy, ox;      // offset of the field in the padded grid
+  int ci;          // workspace lines interleaved (1 or 2, of the row plan)
+  int xr0, xr1, xstep;  // row plan: line b + xstep j of a half holds bin b / xr1 + (b % xr1) xr0 + xstep j
   int nfields;     // fields in this launch
   int group;       // fields per epilogue group (R2 grid.y = ceil(nfields / group))
   int src_group;   // fields sharing one intensity-gradient plane (SRC_INTENSITY)
@@ -68,7 +71,6 @@ struct PassParams {
   int adjoint;     // use conj(H)
   int src_kind;
   int epi_kind;
-  int fp64_r;      // reserved
   int l2_ahead;    // blocks ahead whose input a block prefetches into L2 (0: none)
   uint32_t tune_rows;  // TOP_TUNE_* choices for the row passes (of Mx) and the column pass (of My)
   uint32_t tune_cols;
@@ -121,19 +123,6 @@ struct PassParams {
   unsigned char set_of[kMaxFields];
 };
 
-// Kernel launch timing kinds (instrumentation)
-// Floats per R1 block of the planes staged besides the field rows: the intensity gradient
-// (SRC_INTENSITY) and the phase, amplitude and complex mask of the source modulation.
-__host__ __device__ inline size_t src_plane_floats(const PassParams& p, int rows) {
-  const size_t plane = size_t(rows) * size_t(p.nx);
-  size_t n = 0;
-  if (p.src_kind == SRC_INTENSITY) n += plane;
-  if (p.msrc.flags & TOP_MOD_PHASE) n += plane;
-  if (p.msrc.flags & TOP_MOD_AMPLITUDE) n += plane;
-  if (p.msrc.flags & TOP_MOD_COMPLEX) n += 2 * plane;
-  return n;
-}
-
 // Line transforms of any length P by Bluestein's chirp-z method (padded sizes without a plan of
 // their own): with c[n] = exp(-i pi n^2 / P), the DFT is X[k] = c[k] sum_n (x[n] c[n]) conj(c[k - n]),
 // a convolution done as an L-point FFT (L >= 2P - 1), a product with the transform of the chirp
@@ -177,15 +166,7 @@ void tune_set(int M, uint32_t flags);
 void tune_clear();
 bool tune_save(const char* path, std::string* err);
 bool tune_load(const char* path, std::string* err);
-// Fields per block of the pair-local inverse pass with a field epilogue under tuning flags.
-inline int tune_span(uint32_t flags) {
-  const uint32_t c = (flags >> 8) & 7u;
-  return c == 0 ? 4 : 1 << (c - 1);
-}
-
-// Largest dynamic shared memory of a fused chain block (R2 of one propagation + R1 of the next).
-constexpr size_t kChainSmemMax = 227 * 1024;
-
+// Kernel launch timing kinds (instrumentation)
 enum KernelKind : int { KK_ROWS_FWD = 0, KK_COLS, KK_ROWS_INV, KK_AUX, KK_ROWS_CHAIN, KK_ONCHIP, KK_COUNT };
 
 }  // namespace top
