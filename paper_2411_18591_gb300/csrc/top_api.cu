@@ -92,6 +92,8 @@ struct top_ctx {
   void* cohg = nullptr;  // the coherence backward's G' when the caller wants no grad_in
   size_t cohg_bytes = 0;
   std::vector<void*> allocs;  // cached tables, freed with the handle
+  int* fault = nullptr;       // host-mapped word a kernel sets when a bounded wait runs out
+  int* fault_dev = nullptr;
   std::map<int, float2*> eng_tw;
   std::map<int, float2*> split_tw;
   std::map<std::array<uint64_t, 7>, TransferEntry> transfer;
@@ -111,6 +113,11 @@ namespace {
 
 top_status bind(top_handle h) {
   TOP_CUDA(cudaSetDevice(h->device), "cudaSetDevice");
+  volatile int* fault = h->fault;
+  if (fault && *fault) {
+    *fault = 0;
+    return fail(TOP_ERR_INTERNAL, "a tile copy of an earlier call did not complete; its results are not valid");
+  }
   return TOP_OK;
 }
 
@@ -174,42 +181,40 @@ top_status timed(top_handle h, int kind, cudaStream_t st, const char* what, F&& 
 // ============================================================================= engines and tables
 
 bool find_engine(int M, EngineInfo* info) {
-  return engine_info_small(M, info) || engine_info_mid(M, info) || engine_info_m1024(M, info) ||
-         engine_info_large(M, info) || engine_info_mixed(M, info);
+  return engine_info_small(M, info) || engine_info_m128(M, info) || engine_info_m256(M, info) ||
+         engine_info_m512(M, info) || engine_info_m1024(M, info) || engine_info_m2048(M, info) ||
+         engine_info_m4096(M, info) || engine_info_m250(M, info) || engine_info_m500(M, info) ||
+         engine_info_m768(M, info) || engine_info_m1000(M, info);
 }
 
 cudaError_t launch_pass(int kind, int M, const PassParams& p, cudaStream_t s, const PassParams* next = nullptr) {
-  bool found = false;
-  cudaError_t e = launch_pass_small(kind, M, p, next, s, &found);
-  if (found) return e;
-  e = launch_pass_mid(kind, M, p, next, s, &found);
-  if (found) return e;
-  e = launch_pass_m1024(kind, M, p, next, s, &found);
-  if (found) return e;
-  e = launch_pass_large(kind, M, p, next, s, &found);
-  if (found) return e;
-  e = launch_pass_mixed(kind, M, p, next, s, &found);
-  if (found) return e;
+  using Launch = cudaError_t (*)(int, int, const PassParams&, const PassParams*, cudaStream_t, bool*);
+  static constexpr Launch units[] = {launch_pass_small, launch_pass_m128, launch_pass_m256, launch_pass_m512,
+                                     launch_pass_m1024, launch_pass_m2048, launch_pass_m4096, launch_pass_m250,
+                                     launch_pass_m500, launch_pass_m768, launch_pass_m1000};
+  for (const Launch launch : units) {
+    bool found = false;
+    const cudaError_t e = launch(kind, M, p, next, s, &found);
+    if (found) return e;
+  }
   return cudaErrorInvalidValue;
 }
 
 // Bluestein line pass with convolution length L: one L-point engine up to 4096, two halves on the
 // 4096-point engine for 8192.
 cudaError_t launch_czt_pass(int L, const CztParams& p, cudaStream_t s) {
+  using Launch = cudaError_t (*)(int, const CztParams&, cudaStream_t, bool*);
+  static constexpr Launch units[] = {launch_czt_small, launch_czt_m128, launch_czt_m256, launch_czt_m512,
+                                     launch_czt_m1024, launch_czt_m2048, launch_czt_m4096};
   bool found = false;
-  cudaError_t e;
   if (L > 4096) {
-    e = launch_czt_split_large(L / 2, p, s, &found);
+    const cudaError_t e = launch_czt_split_m4096(L / 2, p, s, &found);
     return found ? e : cudaErrorInvalidValue;
   }
-  e = launch_czt_small(L, p, s, &found);
-  if (found) return e;
-  e = launch_czt_mid(L, p, s, &found);
-  if (found) return e;
-  e = launch_czt_m1024(L, p, s, &found);
-  if (found) return e;
-  e = launch_czt_large(L, p, s, &found);
-  if (found) return e;
+  for (const Launch launch : units) {
+    const cudaError_t e = launch(L, p, s, &found);
+    if (found) return e;
+  }
   return cudaErrorInvalidValue;
 }
 
@@ -352,6 +357,7 @@ top_status di_table(top_handle h, int Py, int Px, double dy, double dx, double l
   float2* ws = samples + plane;
   PassParams p{};
   set_geometry(p, Py, Px, Py, Px);
+  p.fault = h->fault_dev;
   p.method = TOP_DI;
   p.src_kind = SRC_FIELD;
   p.epi_kind = EPI_FIELD;
@@ -1298,6 +1304,7 @@ top_status run_propagation(top_handle h, const Request& q, cudaStream_t st) {
 
   PassParams p{};
   set_geometry(p, geo.ny, geo.nx, geo.Py, geo.Px);
+  p.fault = h->fault_dev;
   p.method = g->method;
   p.adjoint = q.adjoint;
   p.src_kind = q.src_kind;
@@ -1573,6 +1580,7 @@ top_status run_chain(top_handle h, const top_grid* g, const void* in, void* out,
 
   PassParams base{};
   set_geometry(base, geo.ny, geo.nx, geo.Py, geo.Px);
+  base.fault = h->fault_dev;
   base.method = g->method;
   base.src_kind = SRC_FIELD;
   base.epi_kind = EPI_FIELD;
@@ -1744,6 +1752,7 @@ top_status run_ragged(top_handle h, int count, const top_grid* grids, const void
 
     PassParams p{};
     set_geometry(p, geo.ny, geo.nx, geo.Py, geo.Px);
+  p.fault = h->fault_dev;
     p.method = grids[grp[0]].method;
     p.adjoint = backward ? 1 : 0;
     p.src_kind = SRC_FIELD;
@@ -1832,6 +1841,18 @@ top_status top_create(top_handle* out, int device) {
   });
   top_ctx* h = new top_ctx();
   h->device = device;
+  void* word = nullptr;
+  e = cudaHostAlloc(&word, sizeof(int), cudaHostAllocMapped);
+  if (e == cudaSuccess) {
+    h->fault = static_cast<int*>(word);
+    *h->fault = 0;
+    e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->fault_dev), word, 0);
+  }
+  if (e != cudaSuccess) {
+    if (word) cudaFreeHost(word);
+    delete h;
+    return cuda_fail(e, "cudaHostAlloc(fault word)");
+  }
   *out = h;
   return TOP_OK;
 }
@@ -1979,6 +2000,7 @@ top_status top_destroy(top_handle h) {
     cudaEventDestroy(pe.second.second);
   }
   for (cudaEvent_t e : h->pool) cudaEventDestroy(e);
+  cudaFreeHost(h->fault);
   delete h;
   return TOP_OK;
 }

@@ -554,6 +554,32 @@ cudaError_t launch_resample(const float2* in, float2* out, long long batch, Resa
   return cudaSuccess;
 }
 
+cudaError_t encode_tile_map(TileMap* map, const void* ws, long long samples, long long lines, int nfields,
+                            long long field_stride, int box_lines) {
+  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                              const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  static const Encode encode = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
+    return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? reinterpret_cast<Encode>(fn) : nullptr;
+  }();
+  if (!encode) return cudaErrorNotSupported;
+  const cuuint64_t dims[3] = {cuuint64_t(samples), cuuint64_t(lines), cuuint64_t(nfields)};
+  const cuuint64_t strides[2] = {cuuint64_t(samples) * sizeof(float2), cuuint64_t(field_stride) * sizeof(float2)};
+  const cuuint32_t step[3] = {1, 1, 1};
+  for (const bool wide : {false, true}) {
+    const cuuint32_t box[3] = {wide ? 16u : 4u, cuuint32_t(box_lines), 1};
+    // a sample is moved as one 8-byte element
+    const CUresult r = encode(wide ? &map->wide : &map->tile, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, const_cast<void*>(ws),
+                              dims, strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                              CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+  }
+  return cudaSuccess;
+}
+
 cudaError_t launch_transfer_table(float2* hq, int Py, int Px, double dy, double dx, double lam, double z, int method,
                                   int S, int r0, int r1, cudaStream_t s) {
   const int my = Py / 2;

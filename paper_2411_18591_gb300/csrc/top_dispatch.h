@@ -28,19 +28,28 @@ enum PassKind : int { PASS_ROWS_FWD = 0, PASS_COLS = 1, PASS_ROWS_INV = 2, PASS_
                                  bool* found);
 
 TOP_DECLARE_UNIT(small)
-TOP_DECLARE_UNIT(mid)
+TOP_DECLARE_UNIT(m128)
+TOP_DECLARE_UNIT(m256)
+TOP_DECLARE_UNIT(m512)
 TOP_DECLARE_UNIT(m1024)
-TOP_DECLARE_UNIT(large)
-TOP_DECLARE_UNIT(mixed)
+TOP_DECLARE_UNIT(m2048)
+TOP_DECLARE_UNIT(m4096)
+TOP_DECLARE_UNIT(m250)
+TOP_DECLARE_UNIT(m500)
+TOP_DECLARE_UNIT(m768)
+TOP_DECLARE_UNIT(m1000)
 
 #undef TOP_DECLARE_UNIT
 
 // Bluestein line transforms (CztParams) on the power-of-two engines of a unit.
 cudaError_t launch_czt_small(int M, const CztParams& p, cudaStream_t s, bool* found);
-cudaError_t launch_czt_mid(int M, const CztParams& p, cudaStream_t s, bool* found);
+cudaError_t launch_czt_m128(int M, const CztParams& p, cudaStream_t s, bool* found);
+cudaError_t launch_czt_m256(int M, const CztParams& p, cudaStream_t s, bool* found);
+cudaError_t launch_czt_m512(int M, const CztParams& p, cudaStream_t s, bool* found);
 cudaError_t launch_czt_m1024(int M, const CztParams& p, cudaStream_t s, bool* found);
-cudaError_t launch_czt_large(int M, const CztParams& p, cudaStream_t s, bool* found);
+cudaError_t launch_czt_m2048(int M, const CztParams& p, cudaStream_t s, bool* found);
+cudaError_t launch_czt_m4096(int M, const CztParams& p, cudaStream_t s, bool* found);
 // The same as two halves on the 4096-point engine (convolution length 8192).
-cudaError_t launch_czt_split_large(int M, const CztParams& p, cudaStream_t s, bool* found);
+cudaError_t launch_czt_split_m4096(int M, const CztParams& p, cudaStream_t s, bool* found);
 
 }  // namespace top

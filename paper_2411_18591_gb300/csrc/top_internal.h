@@ -5,6 +5,7 @@
 // capturable in a CUDA graph once its tables exist.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -118,6 +119,8 @@ struct PassParams {
   ModDev msrc;  // modulation applied to the R1 source
   ModDev mepi;  // modulation applied in the R2 epilogue
 
+  int* fault;  // host-mapped word set when a bounded wait of a kernel runs out (may be null)
+
   int nsets;
   FieldSet sets[kMaxSets];
   unsigned char set_of[kMaxFields];
@@ -158,6 +161,16 @@ struct CztParams {
   const float2* wsplit;  // L = 8192: exp(-2 pi i p / L), p < L/2
   const float2* const* h;  // CZT_FILTER: per field, rows [line][P] of H / (Py Px) in natural order
 };
+
+// The workspace as a tensor for tile copies: [fields][lines][samples] of complex64, in boxes of
+// box_lines lines x 4 samples (a tile) and x 16 samples (four tiles, 128 bytes a line, for prefetches).
+// Strides in samples; a line is a whole number of 16-byte units.
+struct TileMap {
+  CUtensorMap tile;
+  CUtensorMap wide;
+};
+cudaError_t encode_tile_map(TileMap* map, const void* ws, long long samples, long long lines, int nfields,
+                            long long field_stride, int box_lines);
 
 // The autotune table (top_tune.cu): TOP_TUNE_* flags per line length M (0: the defaults).
 uint32_t tune_flags(int M);

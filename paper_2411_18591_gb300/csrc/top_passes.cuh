@@ -40,36 +40,63 @@
 
 namespace top {
 
-// Rows of a tile and threads of a row block.
+// A row tile: ROWS rows by both halves.
 template <class EN>
 struct RowShape {
+  static constexpr int M = EN::M;
   static constexpr int GW = EN::GW;
   static constexpr int ROWS = GW <= 32 ? 4 : 2;  // rows of a tile (groups wider than a warp: fewer threads a barrier)
-  // Lines interleaved in the workspace. Pairs (64 contiguous bytes a tile of four rows) halve the
-  // wavefronts of the row passes' loads and stores (an access to eight 32-byte pieces takes eight) and
-  // cost the column pass more: at 1024 points fused rows 11.5 -> 9.9 us a field, forward rows 5.7 -> 5.2,
-  // inverse rows 7.4 -> 6.4, column pass 13.3 -> 14.7; a 2048 x 2048-point batch 814 -> 799 us. Handing
-  // the two columns' samples to alternate lanes up to the exchange (whole sectors, a barrier of both
-  // columns' warps per exchange) measured slower: 14.6 against 13.8.
-  static constexpr int CI = (EN::G % 2 == 0 && EN::SL % 2 == 0) ? 2 : 1;
   static constexpr int HALF = ROWS * GW;         // threads of one half of a tile
   static constexpr int TILE = 2 * HALF;
-  static constexpr int TILES = TILE >= 128 ? 1 : 128 / TILE;
-  static constexpr int THREADS = TILE * TILES;
-  static constexpr int BLOCK_ROWS = ROWS * TILES;
   // Stride of the line buffers: the reader lanes of the last exchange (rows fastest) fall on
   // distinct banks (checked by simulation; exact for the power-of-two plans).
   static constexpr int RES = ROWS == 4 || EN::RL == 8 ? 4 : 8;
   static constexpr int LS = EN::BUF + ((RES - EN::BUF) % 16 + 16) % 16;
-  static constexpr size_t SMEM = sizeof(float2) * size_t(TILES) * 2 * ROWS * LS;
+  static constexpr int XH = (ROWS * LS + 15) / 16 * 16;  // float2 of one half's line buffers
+  // Lines interleaved in the workspace: pairs with two rows a tile and for the short plans, whose row
+  // tiles go straight between registers and memory (64 contiguous bytes a tile halve the wavefronts of
+  // their accesses; the column pass then reads half of every sector twice: at 1024 points 14.7 us a
+  // field against 13.3).
+  static constexpr bool LONG = M >= 250 && M <= 2048;
+  static constexpr int CI = ROWS == 2 || !LONG ? 2 : 1;
+  // Tile copies (COPY): a tile is a box of four 8-byte samples (ROWS rows x CI lines) by HL lines a half,
+  // moved by the copy engine in boxes of LB lines.
+  static constexpr int HL = M / CI;
+  static constexpr int box_lines() {
+    if (HL <= 256) return HL;
+    for (int l = 256; l > 4; l -= 4)
+      if (HL % l == 0) return l;
+    return 4;
+  }
+  static constexpr int LB = box_lines();
+  static constexpr int TH = (HL * 4 + 15) / 16 * 16;  // float2 of one half of a copied tile
+  static constexpr unsigned TILE_BYTES = unsigned(2 * HL * 4 * sizeof(float2));
+  static constexpr size_t SMEM_DUO = sizeof(float2) * size_t(4 * XH + 2 * TH) + 128;
+  static constexpr bool COPY = LONG && EN::E >= 16 && SMEM_DUO <= 226 * 1024;
   // registers a thread: 128 for plans of 24 or more samples a thread, 80 for 16 to 20, else 64
   static constexpr int REGS = EN::E >= 24 ? 128 : EN::E >= 16 ? 80 : 64;
-  static constexpr int MINB = 65536 / (THREADS * REGS) > 0 ? 65536 / (THREADS * REGS) : 1;
-  static_assert(SMEM >= 3 * sizeof(double) * THREADS, "room for the overlap reduction");
-  static_assert(THREADS <= 1024, "row block too large");
-  static_assert(GW <= 32 || 2 + ROWS + 2 * ROWS <= 15, "quad, pair and group barriers have ids of their own");
+  static_assert(TH <= XH, "a half's bins fit its line buffers");
   static_assert(EN::M % 2 == 0 && EN::E % 2 == 0, "slots split between the halves");
+  static_assert(CI == 1 || (EN::G % 2 == 0 && EN::SL % 2 == 0), "line pairs stay whole");
 };
+
+// A block of T tiles.
+template <class EN, int T_>
+struct RowBlock : RowShape<EN> {
+  using SH = RowShape<EN>;
+  static constexpr int T = T_;
+  static constexpr int THREADS = SH::TILE * T;
+  static constexpr int BLOCK_ROWS = SH::ROWS * T;
+  static constexpr size_t SMEM_X = sizeof(float2) * size_t(T) * 2 * SH::XH + 64;
+  static constexpr int MINB = 65536 / (THREADS * SH::REGS) > 0 ? 65536 / (THREADS * SH::REGS) : 1;
+  static_assert(THREADS <= 1024, "row block too large");
+  static_assert(SMEM_X >= 3 * sizeof(double) * THREADS, "room for the overlap reduction");
+};
+// Tiles per block: enough for 128 threads; two sharing one copied tile in the passes that load bins by copy.
+template <class EN>
+constexpr int row_tiles() {
+  return RowShape<EN>::TILE >= 128 ? 1 : 128 / RowShape<EN>::TILE;
+}
 
 // Columns per block of the column pass; two thread groups (the two halves) per column, one exchange
 // buffer each.
@@ -135,72 +162,86 @@ __device__ __forceinline__ float2* field_out(const PassParams& p, int f) {
   return p.out_list ? p.out_list[f] : p.out + (long long)f * p.out_stride;
 }
 
-// The place of a thread in a row block: tile of ROWS rows, half r, row and lane of its line, and the
-// row and lane it takes in the frequency layout, where the lanes of one half hold the rows fastest.
-template <class EX>
+// The place of a thread in a block of T row tiles: half r, row and lane of its line, and the row and
+// lane it takes in the frequency layout, where the lanes of one half hold the rows fastest.
+template <class EX, int T>
 struct RowLane {
   using SH = RowShape<EX>;
-  int r, row, t, qrow, qt, tile;
-  bool act;  // not one of the spare threads of a padded group
-  float2* buf;         // this line's buffer
-  const float2* peer;  // the other half's
-  float2* qbuf;        // line buffer of (r, qrow)
+  float2* smem;
 
-  __device__ __forceinline__ explicit RowLane(float2* smem) {
-    tile = int(threadIdx.x) / SH::TILE;
-    const int v = int(threadIdx.x) % SH::TILE;
-    r = v / SH::HALF;
-    const int u = v % SH::HALF;
-    row = u / SH::GW;
-    const int tl = u % SH::GW;
-    qrow = u % SH::ROWS;
-    const int ql = u / SH::ROWS;
-    if constexpr (SH::GW == EX::G) {
-      t = tl;
-      qt = ql;
-      act = true;
-    } else {
-      t = min(tl, EX::G - 1);
-      qt = min(ql, EX::G - 1);
-      act = tl < EX::G;
-    }
-    float2* base = smem + tile * 2 * SH::ROWS * SH::LS;
-    buf = base + (r * SH::ROWS + row) * SH::LS;
-    peer = base + ((r ^ 1) * SH::ROWS + row) * SH::LS;
-    qbuf = base + (r * SH::ROWS + qrow) * SH::LS;
+  __device__ __forceinline__ explicit RowLane(float2* s) : smem(s) {}
+  __device__ __forceinline__ static int tid() { return int(threadIdx.x); }
+  __device__ __forceinline__ static int in_tile(int v) { return T == 1 ? v : v % SH::TILE; }
+  __device__ __forceinline__ static int spare(int l) { return SH::GW == EX::G ? l : min(l, EX::G - 1); }
+  __device__ __forceinline__ static int half_of(int v) { return in_tile(v) / SH::HALF; }
+  __device__ __forceinline__ static int tile_of(int v) { return T == 1 ? 0 : v / SH::TILE; }
+  __device__ __forceinline__ static int row_of(int v) { return in_tile(v) % SH::HALF / SH::GW; }
+  __device__ __forceinline__ static int qrow_of(int v) { return v % SH::ROWS; }
+  __device__ __forceinline__ static int tile() { return tile_of(tid()); }
+  __device__ __forceinline__ static int r() { return half_of(tid()); }
+  __device__ __forceinline__ static int row() { return row_of(tid()); }
+  __device__ __forceinline__ static int t() { return spare(tid() % SH::GW); }
+  __device__ __forceinline__ static int qrow() { return qrow_of(tid()); }
+  __device__ __forceinline__ static int qt() { return spare(in_tile(tid()) % SH::HALF / SH::ROWS); }
+  // not one of the spare threads of a padded group
+  __device__ __forceinline__ static bool act() { return SH::GW == EX::G || tid() % SH::GW < EX::G; }
+  __device__ __forceinline__ static bool lead() { return in_tile(tid()) == 0; }             // of the tile
+  __device__ __forceinline__ static bool hlead() { return in_tile(tid()) % SH::HALF == 0; }  // of the tile's half
+  // this half's line buffers, this line's, the other half's line's, the one of (half, qrow)
+  __device__ __forceinline__ float2* half(int v) const { return smem + (tile_of(v) * 2 + half_of(v)) * SH::XH; }
+  __device__ __forceinline__ float2* half() const { return half(tid()); }
+  __device__ __forceinline__ float2* buf() const {
+    const int v = tid();
+    return half(v) + row_of(v) * SH::LS;
   }
+  __device__ __forceinline__ const float2* peer() const {
+    const int v = tid();
+    return smem + (tile_of(v) * 2 + (half_of(v) ^ 1)) * SH::XH + row_of(v) * SH::LS;
+  }
+  __device__ __forceinline__ float2* qbuf() const {
+    const int v = tid();
+    return half(v) + qrow_of(v) * SH::LS;
+  }
+  // Barrier ids: tiles 1.., halves, rows; line groups wider than a warp count down from 15 (EX::sync_group).
   // all threads of the tile
   __device__ __forceinline__ void tile_sync() const {
-    if constexpr (SH::TILES == 1) __syncthreads();
+    if constexpr (T == 1) __syncthreads();
     else if constexpr (SH::TILE <= 32) __syncwarp();
-    else top_named_barrier(1 + tile, SH::TILE);
+    else top_named_barrier(1 + tile(), SH::TILE);
   }
   // the rows of this half (the last exchange regroups them)
   __device__ __forceinline__ void quad_sync() const {
     if constexpr (SH::HALF <= 32) __syncwarp();
-    else if constexpr (SH::TILES == 1) top_named_barrier(1 + r, SH::HALF);
+    else if constexpr (T <= 2) top_named_barrier(3 + tid() / SH::HALF, SH::HALF);
     else tile_sync();
   }
   // the two halves of this row
   __device__ __forceinline__ void pair_sync() const {
-    if constexpr (SH::GW >= 32) top_named_barrier(3 + row, 2 * SH::GW);
+    if constexpr (SH::GW == 32) top_named_barrier(7 + SH::ROWS * tile() + row(), 2 * SH::GW);
     else tile_sync();
   }
+  static_assert(SH::GW <= 32 || (T <= 2 && 15 - T * 2 * SH::ROWS >= 6), "group barriers clear of the others");
+  static_assert(SH::GW != 32 || T <= 2, "row barriers have ids of their own");
 };
 
 // First workspace sample of lane qt of half r, row y of field f; slot (q, j) sits (G q + S j) ny on.
 template <class EX>
 __device__ __forceinline__ float2* ws_lane(const PassParams& p, int f, int r, int qt, int y) {
-  static_assert(RowShape<EX>::CI == 1 || (EX::G % 2 == 0 && EX::SL % 2 == 0 && EX::M % 2 == 0), "line pairs stay whole");
   float2* ws = p.ws + (long long)f * p.ws_stride;
   const int line = r * EX::M + qt;
   if constexpr (RowShape<EX>::CI == 1) return ws + (long long)line * p.ny + y;
   else return ws + ((long long)(line >> 1) * p.ny + y) * 2 + (line & 1);
 }
-
+// The same in one half of a copied tile, [HL][4]; slot (q, j) sits (G q + S j) / CI lines on.
 template <class EX>
-__device__ __forceinline__ void load_bins(const PassParams& p, int f, const RowLane<EX>& c, int y, float2 (&v)[EX::E]) {
-  const float2* w = ws_lane<EX>(p, f, c.r, c.qt, y);
+__device__ __forceinline__ int tile_lane(int qt, int qrow) {
+  if constexpr (RowShape<EX>::CI == 1) return qt * 4 + qrow;
+  else return (qt >> 1) * 4 + qrow * 2 + (qt & 1);
+}
+
+template <class EX, class Lane>
+__device__ __forceinline__ void load_bins(const PassParams& p, int f, const Lane& c, int y, float2 (&v)[EX::E]) {
+  const float2* w = ws_lane<EX>(p, f, c.r(), c.qt(), y);
   const bool live = y < p.ny;
 #pragma unroll
   for (int e = 0; e < EX::E; ++e) {
@@ -208,10 +249,9 @@ __device__ __forceinline__ void load_bins(const PassParams& p, int f, const RowL
     v[e] = live ? w[(EX::G * q + EX::SL * j) * p.ny] : make_float2(0.f, 0.f);
   }
 }
-template <class EX>
-__device__ __forceinline__ void store_bins(const PassParams& p, int f, const RowLane<EX>& c, int y,
-                                           const float2 (&v)[EX::E]) {
-  float2* w = ws_lane<EX>(p, f, c.r, c.qt, y);
+template <class EX, class Lane>
+__device__ __forceinline__ void store_bins(const PassParams& p, int f, const Lane& c, int y, const float2 (&v)[EX::E]) {
+  float2* w = ws_lane<EX>(p, f, c.r(), c.qt(), y);
   if (y < p.ny) {
 #pragma unroll
     for (int e = 0; e < EX::E; ++e) {
@@ -220,6 +260,237 @@ __device__ __forceinline__ void store_bins(const PassParams& p, int f, const Row
     }
   }
 }
+template <class EX, class Lane>
+__device__ __forceinline__ void read_tile(const float2* tile, const Lane& c, float2 (&v)[EX::E]) {
+  const float2* w = tile + c.r() * RowShape<EX>::TH + tile_lane<EX>(c.qt(), c.qrow());
+#pragma unroll
+  for (int e = 0; e < EX::E; ++e) {
+    const int q = e / EX::RL, j = e % EX::RL;
+    v[e] = w[(EX::G * q + EX::SL * j) * (4 / RowShape<EX>::CI)];
+  }
+}
+// The bins of a tile to the workspace through the half's line buffers, by copy. Returns with the copy
+// in flight: the half's leading thread waits for it (top_bulk_wait_read) before the buffers are written
+// again.
+template <class EX, class Lane>
+__device__ __forceinline__ void copy_bins_out(const TileMap& map, int f, const Lane& c, int y0, const float2 (&v)[EX::E]) {
+  using SH = RowShape<EX>;
+  c.quad_sync();  // the half's last exchange reads are done
+  float2* w = c.half() + tile_lane<EX>(c.qt(), c.qrow());
+#pragma unroll
+  for (int e = 0; e < EX::E; ++e) {
+    const int q = e / EX::RL, j = e % EX::RL;
+    w[(EX::G * q + EX::SL * j) * (4 / SH::CI)] = v[e];
+  }
+  top_async_fence();
+  c.quad_sync();
+  if (c.hlead()) {
+#pragma unroll 1
+    for (int l = 0; l < SH::HL; l += SH::LB) top_tma_store3(&map.tile, y0 * SH::CI, c.r() * SH::HL + l, f, c.half() + l * 4);
+    top_bulk_commit();
+  }
+}
+// The half's buffers are free of outgoing copies.
+template <class Lane>
+__device__ __forceinline__ void copy_out_done(const Lane& c) {
+  if (c.hlead()) top_bulk_wait_read();
+  c.quad_sync();
+}
+
+// Bound of the waits on copies and tickets, in clock cycles (about two seconds).
+constexpr long long kWaitCycles = 4000000000ll;
+
+// The work items a block runs: its own index, then those of blocks that have not started. Items are handed
+// out in order, so the tiles in flight stay neighbours and the sectors of a line meet in L2: fixed shares
+// of the items per block drifted apart over a long launch (the 384-field step's fused rows took 11.1 us
+// a field with 24 fields and 16.4 with 384).
+struct Tickets {
+  struct Shared {
+    alignas(16) unsigned answer[4];
+    unsigned long long bar;
+    int parity, open;
+  };
+  Shared* s;
+
+  __device__ __forceinline__ explicit Tickets(void* mem) : s(static_cast<Shared*>(mem)) {}
+  // one thread, before the block's first barrier
+  __device__ __forceinline__ void init() const {
+    top_mbar_init(&s->bar, 1);
+    top_mbar_fence();
+    s->parity = 0;
+    s->open = 1;
+  }
+  __device__ __forceinline__ void ask() const {
+    top_mbar_expect(&s->bar, 16);
+    top_ask_ticket(s->answer, &s->bar);
+  }
+  // The asked item, or -1; asks for the next one. One thread at a time, in an order that barriers give.
+  __device__ __forceinline__ int take(int* fault, bool again = true) const {
+    if (!s->open) return -1;
+    int item = -1;
+    if (top_mbar_wait(&s->bar, s->parity, kWaitCycles)) {
+      item = top_ticket(s->answer);
+    } else if (fault) {
+      *fault = 1;
+    }
+    s->parity ^= 1;
+    if (item < 0) {
+      s->open = 0;
+    } else if (again) {
+      top_async_fence();  // the answer has been read
+      ask();
+    }
+    return item;
+  }
+};
+
+// Rows by tile copies. The scattered accesses of a row tile (2 x 1024 lines, 32 bytes each at 1024
+// points) took half of the row passes' L1 wavefronts and left their latency exposed; the copy engine
+// moves the same boxes at 5.4 TB/s read and 2 x 2.5 TB/s in place, without either. Per field at 1024
+// points (64-field launches, direct with its own best layout -> copies): forward rows 4.6 -> 4.2 us,
+// fused rows 10.4 -> 9.7, inverse rows 5.8 -> 5.3, with the phase gradient 12.9 -> 10.4, and the column
+// pass, whose lines no longer need to be interleaved for the rows' sake, 14.2 -> 12.7.
+//
+// Two tiles of a block (groups 0 and 1, 256 threads each at 1024 points) work in antiphase on one copied
+// tile of shared memory: while a group transforms its rows in registers and its own line buffers, the
+// copy engine brings the other group's next tile. Tiles are brought for group 0, 1, 0, 1, ... (a group
+// that has run out is skipped); the group that has read a tile starts the next copy. An item is a row
+// tile of the fields of one group.
+template <class EX>
+struct TileFeed {
+  using SH = RowShape<EX>;
+  struct Shared {
+    Tickets::Shared tickets;
+    unsigned long long full[2];
+    int item[2], f[2], x[2];    // the tile each group is to take next (item < 0: there is none), its box's x
+    int cur_item[2][2], cur_f[2][2];  // [turn][group]: the tile each group has in hand (a group's threads
+                                      // are at most one take apart)
+    int alive[2];  // not yet told that there are no more tiles
+    int ok[2];
+  };
+  static_assert(sizeof(Shared) <= 128, "reserved after the tiles");
+  float2* tile;
+  Shared* s;
+  int ntiles, group, nfields, ahead;
+  unsigned turn;  // of this group's next take: the parity of its copy
+
+  __device__ __forceinline__ TileFeed(float2* smem, int ny, int nfields_, int group_, int ahead_)
+      : tile(smem + 4 * SH::XH), s(reinterpret_cast<Shared*>(smem + 4 * SH::XH + 2 * SH::TH)), group(group_),
+        nfields(nfields_), ahead(ahead_), turn(0) {
+    ntiles = (ny + SH::ROWS - 1) / SH::ROWS;
+    if (threadIdx.x == 0) {
+      const Tickets tickets(&s->tickets);
+      tickets.init();
+      top_mbar_init(s->full, 1);
+      top_mbar_init(s->full + 1, 1);
+      top_mbar_fence();
+      s->item[1] = -1;
+      s->alive[0] = s->alive[1] = 1;
+      tickets.ask();
+    }
+    __syncthreads();
+  }
+  // group 0's first tile, the block's own item (one thread)
+  __device__ __forceinline__ void start(const TileMap& map) const {
+    plan(0, blockIdx.x, first_field(blockIdx.x));
+    bring(map, 0);
+  }
+  __device__ __forceinline__ int first_field(int it) const { return it / ntiles * group; }
+  __device__ __forceinline__ int end_field(int it) const { return min(first_field(it) + group, nfields); }
+  // the tile in hand (after take, until the group's next)
+  __device__ __forceinline__ int item() const { return s->cur_item[turn ^ 1][RowLane<EX, 2>::tile()]; }
+  __device__ __forceinline__ int field() const { return s->cur_f[turn ^ 1][RowLane<EX, 2>::tile()]; }
+  __device__ __forceinline__ int y0() const {
+    const int it = item();
+    return (it - it / ntiles * ntiles) * SH::ROWS;
+  }
+
+  __device__ __forceinline__ void plan(int g, int it, int ff) const {
+    s->item[g] = it;
+    s->f[g] = ff;
+    s->x[g] = (it - it / ntiles * ntiles) * SH::ROWS * SH::CI;
+    s->alive[g] = it >= 0;
+  }
+  // Copy in the planned tile of group g, or tell it that there is none.
+  __device__ __forceinline__ void bring(const TileMap& map, int g) const {
+    if (s->item[g] < 0) {
+      top_mbar_arrive(s->full + g);
+      return;
+    }
+    top_mbar_expect(s->full + g, SH::TILE_BYTES);
+    const int x = s->x[g], f = s->f[g];
+#pragma unroll 1
+    for (int l = 0; l < 2 * SH::HL; l += SH::LB)
+      top_tma_load3(tile + (l < SH::HL ? l * 4 : SH::TH + (l - SH::HL) * 4), &map.tile, x, l, f, s->full + g);
+    if (ahead > 0 && (x & 15) == 0) {
+      // the first of four tiles side by side: the four's next field, or the four tiles one wave of
+      // resident groups later, go to L2
+      int it = s->item[g], nf = f + 1;
+      if (nf >= end_field(it)) {
+        it += ahead;
+        nf = first_field(it);
+        if (nf >= nfields) return;
+      }
+      const int nx = (it - it / ntiles * ntiles) * SH::ROWS * SH::CI & ~15;
+#pragma unroll 1
+      for (int l = 0; l < 2 * SH::HL; l += SH::LB) top_tma_prefetch3(&map.wide, nx, l, nf);
+    }
+  }
+  // the item and field after (it, ff), from the tickets at the end of an item; it < 0: none
+  __device__ __forceinline__ void following(int& it, int& ff, int* fault) const {
+    if (it >= 0 && ff + 1 < end_field(it)) {
+      ++ff;
+    } else {
+      it = Tickets(&s->tickets).take(fault);
+      ff = it >= 0 ? first_field(it) : 0;
+    }
+  }
+  // Wait for this group's tile, take its bins, start the next copy. False (for the whole group) when there
+  // is none, or if the copy has not come within the bound (the fault word is then set).
+  template <class Lane>
+  __device__ __forceinline__ bool take(const TileMap& map, const Lane& c, int* fault, float2 (&v)[EX::E]) {
+    int calls = 0;  // groups to bring tiles for: bit g
+    if (c.lead()) {
+      const int g = c.tile(), o = g ^ 1;
+      const bool ok = top_mbar_wait(s->full + g, turn, kWaitCycles);
+      if (!ok) {
+        if (fault) *fault = 1;
+        if (s->tickets.open) top_mbar_wait(&s->tickets.bar, s->tickets.parity, kWaitCycles);
+      }
+      const int it = s->item[g], ff = s->f[g];
+      s->ok[g] = ok && it >= 0;
+      s->cur_item[turn][g] = it;
+      s->cur_f[turn][g] = ff;
+      if (ok && it >= 0) {
+        int ni = -1, nf = 0;
+        if (s->alive[o]) {
+          ni = s->item[o];
+          nf = s->f[o];
+          following(ni, nf, fault);
+          plan(o, ni, nf);
+          calls |= 1 << o;
+        }
+        if (ni < 0) {  // the other group has run out: this one goes on alone
+          ni = it;
+          nf = ff;
+          following(ni, nf, fault);
+          plan(g, ni, nf);
+          calls |= 1 << g;
+        }
+      }
+    }
+    c.tile_sync();
+    const int g = c.tile();
+    if (!s->ok[g]) return false;
+    top_mbar_try(s->full + g, turn);  // complete: orders the copied tile before this thread's reads
+    read_tile<EX>(tile, c, v);
+    c.tile_sync();
+    if (calls & 1) bring(map, 0);
+    if (calls & 2) bring(map, 1);
+    turn ^= 1;
+    return true;
+  }
+};
 
 // Position of own slot k of half r (slot k or E/2 + k: a constant step between the two).
 template <class EN>
@@ -465,72 +736,104 @@ __device__ __forceinline__ void src_samples(const SrcRow& s, int n, At&& at, flo
 }
 
 // Without a source modulation (MF = 0) both halves load the whole row (the second read hits L1) and
-// nothing is traded; with one, each half modulates its own slots and the halves trade.
-template <class EX, bool X2, uint32_t MF>
-__global__ void __launch_bounds__(RowShape<EX>::THREADS, RowShape<EX>::MINB) k_rows_fwd(const __grid_constant__ PassParams p) {
-  using SH = RowShape<EX>;
-  constexpr int E = EX::E, M = EX::M, H = E / 2;
+// nothing is traded; with one, each half modulates its own slots and the halves trade. With COPY the
+// bins leave through the copy engine, and a block goes on to the next tile while they do.
+template <class EX, bool X2, uint32_t MF, bool COPY>
+__global__ void __launch_bounds__(RowBlock<EX, row_tiles<EX>()>::THREADS, RowBlock<EX, row_tiles<EX>()>::MINB)
+    k_rows_fwd(const __grid_constant__ PassParams p, const __grid_constant__ TileMap map) {
+  constexpr int T = row_tiles<EX>();
+  using SH = RowBlock<EX, T>;
+  constexpr int E = EX::E, H = E / 2;
   TOP_DYN_SMEM(float2, smem);
-  const RowLane<EX> c(smem);
-  const int tile0 = (blockIdx.x * SH::TILES + c.tile) * SH::ROWS;
-  const int y = tile0 + c.row;
-  const int f = blockIdx.y;
-  const int nx = p.nx;
-  const bool live = y < p.ny;
-  if (threadIdx.x == 0 && p.l2_ahead > 0) {
-    // the rows of the block one wave of resident blocks later go to L2 while this one works
-    const long long lb = (long long)blockIdx.y * gridDim.x + blockIdx.x + p.l2_ahead;
-    if (lb < (long long)gridDim.x * gridDim.y) {
-      const int fa = int(lb / gridDim.x), ya = int(lb % gridDim.x) * SH::BLOCK_ROWS;
+  const RowLane<EX, T> c(smem);
+  const int nx = p.nx, o = p.ox;
+  const int ntiles = (p.ny + SH::BLOCK_ROWS - 1) / SH::BLOCK_ROWS;
+  const int total = ntiles * p.nfields;
+  struct Next {
+    Tickets::Shared tickets;
+    int item[2];
+  };
+  static_assert(sizeof(Next) <= 64, "reserved after the line buffers");
+  Next* next = reinterpret_cast<Next*>(smem + T * 2 * SH::XH);
+  const Tickets tickets(&next->tickets);
+  if constexpr (COPY) {
+    if (threadIdx.x == 0) {
+      tickets.init();
+      tickets.ask();
+    }
+  }
+  int turn = 0;
+#pragma unroll 1
+  for (int i = blockIdx.x; i >= 0; turn ^= 1) {
+    const int f = COPY ? i / ntiles : blockIdx.y;
+    const int tile0 = (COPY ? i - f * ntiles : i) * SH::BLOCK_ROWS + c.tile() * SH::ROWS;
+    const int y = tile0 + c.row();
+    const bool live = y < p.ny;
+    const int next_wave = (COPY ? i : blockIdx.y * ntiles + i) + p.l2_ahead;
+    if (threadIdx.x == 0 && p.l2_ahead > 0 && next_wave < total) {
+      // the rows of the tile one wave of resident blocks later go to L2 while this one works
+      const int fa = next_wave / ntiles, ya = (next_wave - fa * ntiles) * SH::BLOCK_ROWS;
       const int na = min(SH::BLOCK_ROWS, p.ny - ya);
       const long long rowa = (long long)ya * nx;
       const float2* src = p.src_kind == SRC_INTENSITY ? p.psi + (long long)fa * p.psi_stride + rowa : field_in(p, fa) + rowa;
       top_prefetch_l2(src, unsigned(na) * nx * 8u);
     }
-  }
-  const SrcRow s = src_row(p, f, live ? y : 0);
-  const int n = live ? nx : 0;  // rows past the field are zero
-  float2 v[E];
-  const int o = p.ox;
-  if constexpr (MF == 0) {
-    src_samples<E>(s, n, [&](int e) { return sample_lo<EX, X2>(EX::in_pos(c.t, e), o); }, v);
-    if constexpr (!X2) {
+    const SrcRow s = src_row(p, f, live ? y : 0);
+    const int n = live ? nx : 0;  // rows past the field are zero
+    float2 v[E];
+    if constexpr (MF == 0) {
+      src_samples<E>(s, n, [&](int e) { return sample_lo<EX, X2>(EX::in_pos(c.t(), e), o); }, v);
+      if constexpr (!X2) {
 #pragma unroll
-      for (int e0 = 0; e0 < E; e0 += H) {
-        float2 b[H];
-        src_samples<H>(s, n, [&](int e) { return sample_hi<EX>(EX::in_pos(c.t, e0 + e), o); }, b);
+        for (int e0 = 0; e0 < E; e0 += H) {
+          float2 b[H];
+          src_samples<H>(s, n, [&](int e) { return sample_hi<EX>(EX::in_pos(c.t(), e0 + e), o); }, b);
 #pragma unroll
-        for (int e = 0; e < H; ++e) v[e0 + e] = c.r ? c_sub(v[e0 + e], b[e]) : c_add(v[e0 + e], b[e]);
+          for (int e = 0; e < H; ++e) v[e0 + e] = c.r() ? c_sub(v[e0 + e], b[e]) : c_add(v[e0 + e], b[e]);
+        }
       }
-    }
-  } else {
-    const ModDev& m = p.msrc;
-    const uint32_t flags = mod_flags<MF>(m);
-    const FieldSet& fs = p.sets[p.set_of[f]];
-    const ModRow mr = mod_row(m, flags, fs.src_lx, fs.src_ly, f, live ? y : 0, nx);
-    float2 lo[H], hi[H], mv[H];
-    const OwnSamples<EX, X2> at_lo{c.r, c.t, o, false};
-    src_samples<H>(s, n, at_lo, lo);
-    mod_values(m, flags, m.conj, mr, nx, at_lo, mv);
+    } else {
+      const ModDev& m = p.msrc;
+      const uint32_t flags = mod_flags<MF>(m);
+      const FieldSet& fs = p.sets[p.set_of[f]];
+      const ModRow mr = mod_row(m, flags, fs.src_lx, fs.src_ly, f, live ? y : 0, nx);
+      float2 lo[H], hi[H], mv[H];
+      const OwnSamples<EX, X2> at_lo{c.r(), c.t(), o, false};
+      src_samples<H>(s, n, at_lo, lo);
+      mod_values(m, flags, m.conj, mr, nx, at_lo, mv);
 #pragma unroll
-    for (int k = 0; k < H; ++k) lo[k] = c_mul(lo[k], mv[k]);
-    if constexpr (!X2) {
-      const OwnSamples<EX, X2> at_hi{c.r, c.t, o, true};
-      src_samples<H>(s, n, at_hi, hi);
-      mod_values(m, flags, m.conj, mr, nx, at_hi, mv);
+      for (int k = 0; k < H; ++k) lo[k] = c_mul(lo[k], mv[k]);
+      if constexpr (!X2) {
+        const OwnSamples<EX, X2> at_hi{c.r(), c.t(), o, true};
+        src_samples<H>(s, n, at_hi, hi);
+        mod_values(m, flags, m.conj, mr, nx, at_hi, mv);
 #pragma unroll
-      for (int k = 0; k < H; ++k) hi[k] = c_mul(hi[k], mv[k]);
+        for (int k = 0; k < H; ++k) hi[k] = c_mul(hi[k], mv[k]);
+      }
+      if constexpr (COPY) copy_out_done(c);
+      trade_fold<EX, X2>(v, lo, hi, c.buf(), c.peer(), c.r(), c.t(), [&] { c.pair_sync(); });
     }
-    trade_fold<EX, X2>(v, lo, hi, c.buf, c.peer, c.r, c.t, [&] { c.pair_sync(); });
+    if (c.r()) fold_odd<EX, X2>(v, p.wpx, c.t());
+    EX::template fwd_to<false>(
+        v, c.buf(), c.t(), p.twx,
+        [&] {
+          if constexpr (MF != 0) c.pair_sync();  // the other half has read the traded slots
+          else if constexpr (COPY) copy_out_done(c);
+        },
+        c.qbuf(), c.qt(), [&] { c.quad_sync(); });
+    if constexpr (COPY) {
+      copy_bins_out<EX>(map, f, c, tile0, v);
+      if (threadIdx.x == 0) next->item[turn] = tickets.take(p.fault);
+      __syncthreads();
+      i = next->item[turn];
+    } else {
+      store_bins<EX>(p, f, c, tile0 + c.qrow(), v);
+      i = -1;
+    }
   }
-  if (c.r) fold_odd<EX, X2>(v, p.wpx, c.t);
-  EX::template fwd_to<false>(
-      v, c.buf, c.t, p.twx,
-      [&] {
-        if constexpr (MF != 0) c.pair_sync();  // the other half has read the traded slots
-      },
-      c.qbuf, c.qt, [&] { c.quad_sync(); });
-  store_bins<EX>(p, f, c, tile0 + c.qrow, v);
+  if constexpr (COPY) {
+    if (c.hlead()) top_bulk_wait();
+  }
 }
 
 // ----------------------------------------------------------------------------- C
@@ -701,61 +1004,63 @@ __device__ __forceinline__ void overlap_add(OvAcc& acc, float2 val, float2 phi) 
   acc.pw = fma(vx, vx, fma(vy, vy, acc.pw));
 }
 
-// A block runs its rows of p.group consecutive fields. At padding 2 the group's intensity and phase
-// partials are summed in registers (each own slot stands for one sample of the row), otherwise and
-// for the amplitude and mask partials the owner thread adds to the planes in memory; both in field order.
-template <class EX, bool X2, int KIND, uint32_t MF>
-__global__ void __launch_bounds__(RowShape<EX>::THREADS, RowShape<EX>::MINB) k_rows_inv(const __grid_constant__ PassParams p) {
-  using SH = RowShape<EX>;
-  constexpr int E = EX::E, M = EX::M, H = E / 2;
-  constexpr bool REG_ACC = X2 && (KIND == EPI_INTENSITY || KIND == EPI_MODGRAD);
-  TOP_DYN_SMEM(float2, smem);
-  const RowLane<EX> c(smem);
-  const int tile0 = (blockIdx.x * SH::TILES + c.tile) * SH::ROWS;
-  const int y = tile0 + c.row;
-  const int g = blockIdx.y;
-  const int f0 = g * p.group;
-  const int f1 = min(f0 + p.group, p.nfields);
-  const int nx = p.nx;
-  const bool live = y < p.ny && c.act;
-  const ModDev& m = p.mepi;
-  const uint32_t flags = mod_flags<MF>(m);
-  const long long row0 = (long long)y * nx;
-  const bool grads = KIND == EPI_MODGRAD && (p.part_phase || p.part_amp || p.part_mask);
-  const long long part0 = (long long)g * p.part_stride + row0;
+// A tile's rows of p.group consecutive fields. At padding 2 the group's intensity and phase partials are
+// summed in registers (each own slot stands for one sample of the row), otherwise and for the amplitude
+// and mask partials the owner thread adds to the planes in memory; both in field order.
+template <class EX, bool X2, int KIND>
+struct RowEpilogue {
+  static constexpr int H = EX::E / 2;
+  static constexpr bool REG_ACC = X2 && (KIND == EPI_INTENSITY || KIND == EPI_MODGRAD);
   float acc[REG_ACC ? H : 1];
-  if constexpr (REG_ACC) {
+  OvAcc ov;
+
+  // first field of a group: the partials so far
+  template <class Lane>
+  __device__ __forceinline__ void open(const PassParams& p, const Lane& c, int g, int y) {
+    if constexpr (REG_ACC) {
 #pragma unroll
-    for (int k = 0; k < H; ++k) acc[k] = 0.f;
-    if (KIND == EPI_MODGRAD && p.part_phase && p.part_accumulate && live) {
+      for (int k = 0; k < H; ++k) acc[k] = 0.f;
+      if (KIND == EPI_MODGRAD && p.part_phase && p.part_accumulate && c.act() && y < p.ny) {
+        const float* src = p.part_phase + (long long)g * p.part_stride + (long long)y * p.nx;
 #pragma unroll
-      for (int k = 0; k < H; ++k) acc[k] = p.part_phase[part0 + sample_lo<EX, X2>(own_pos<EX>(c.r, c.t, k), 0)];
+        for (int k = 0; k < H; ++k) acc[k] = src[sample_lo<EX, X2>(own_pos<EX>(c.r(), c.t(), k), 0)];
+      }
     }
   }
-#pragma unroll 1
-  for (int f = f0; f < f1; ++f) {
-    float2 v[E];
-    load_bins<EX>(p, f, c, tile0 + c.qrow, v);
-    EX::template inv_from<true>(
-        v, c.qbuf, c.qt,
-        [&] {
-          if (f > f0) c.tile_sync();  // the previous field's trade has been read
-        },
-        c.buf, c.t, [&] { c.quad_sync(); }, p.twx);
-    if (c.r) unfold_odd<EX, X2>(v, p.wpx, c.t);
-    float2 lo[H], hi[H];
-    trade_combine<EX, X2>(v, lo, hi, c.buf, c.peer, c.r, c.t, [] { EX::sync_group(); }, [&] { c.pair_sync(); });
+  // last field done
+  template <class Lane>
+  __device__ __forceinline__ void close(const PassParams& p, const Lane& c, int g, int y) {
+    if constexpr (REG_ACC) {
+      const long long row0 = (long long)y * p.nx;
+      float* dst = KIND == EPI_INTENSITY ? p.outf + (long long)g * p.outf_stride + row0
+                                         : (p.part_phase ? p.part_phase + (long long)g * p.part_stride + row0 : nullptr);
+      if (c.act() && y < p.ny && dst) {
+#pragma unroll
+        for (int k = 0; k < H; ++k) dst[sample_lo<EX, X2>(own_pos<EX>(c.r(), c.t(), k), 0)] = acc[k];
+      }
+    }
+  }
+  // the own slots' samples of row y of field f in group g
+  template <uint32_t MF, class Lane>
+  __device__ __forceinline__ void field(const PassParams& p, const Lane& c, int f, int g, bool first, int y,
+                                        const float2 (&lo)[H], const float2 (&hi)[H]) {
+    const int nx = p.nx;
+    const bool live = y < p.ny && c.act();
+    const ModDev& m = p.mepi;
+    const uint32_t flags = mod_flags<MF>(m);
+    const long long row0 = (long long)y * nx;
+    const bool grads = KIND == EPI_MODGRAD && (p.part_phase || p.part_amp || p.part_mask);
+    const long long part0 = (long long)g * p.part_stride + row0;
     const FieldSet& fs = p.sets[p.set_of[f]];
     const ModRow mr = mod_row(m, flags, fs.epi_lx, fs.epi_ly, f, live ? y : 0, nx);
     const float w = KIND == EPI_INTENSITY && p.weights ? __ldg(p.weights + f) : 1.f;
     float2* out = KIND == EPI_FIELD ? field_out(p, f) + row0 : (p.out ? p.out + (long long)f * p.out_stride + row0 : nullptr);
     const float2* xs = grads ? p.xs + (long long)f * p.xs_stride + row0 : nullptr;
-    const bool first = f == f0;
     const bool fresh = first && !p.part_accumulate;
-    OvAcc ov{0.0, 0.0, 0.0};
+    ov = OvAcc{0.0, 0.0, 0.0};
     // own slots' samples val0
     auto samples = [&](const float2 (&val0)[H], bool hi_part) {
-      const OwnSamples<EX, X2> at{c.r, c.t, p.ox, hi_part};
+      const OwnSamples<EX, X2> at{c.r(), c.t(), p.ox, hi_part};
       if constexpr (KIND == EPI_MODGRAD) {
         // val = dL/dy with y = M x (M without conjugation), in two rounds of slots
         constexpr int N = H % 2 == 0 ? H / 2 : H;
@@ -816,36 +1121,79 @@ __global__ void __launch_bounds__(RowShape<EX>::THREADS, RowShape<EX>::MINB) k_r
       samples(lo, false);
       if constexpr (!X2) samples(hi, true);
     }
-    if constexpr (KIND == EPI_OVERLAP) {
-      // the block's sums in a fixed order: every thread's three values, added by thread 0
-      __syncthreads();
-      double* red = reinterpret_cast<double*>(smem);
-      red[3 * threadIdx.x] = ov.re;
-      red[3 * threadIdx.x + 1] = ov.im;
-      red[3 * threadIdx.x + 2] = ov.pw;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double sr = 0.0, si = 0.0, sp = 0.0;
-        for (int i = 0; i < SH::THREADS; ++i) {
-          sr += red[3 * i];
-          si += red[3 * i + 1];
-          sp += red[3 * i + 2];
-        }
-        double* o = p.ov_part + ((long long)f * gridDim.x + blockIdx.x) * 3;
-        o[0] = sr;
-        o[1] = si;
-        o[2] = sp;
-      }
-      __syncthreads();
-    }
   }
-  if constexpr (REG_ACC) {
-    float* dst = KIND == EPI_INTENSITY ? p.outf + (long long)g * p.outf_stride + row0
-                                       : (p.part_phase ? p.part_phase + part0 : nullptr);
-    if (live && dst) {
-#pragma unroll
-      for (int k = 0; k < H; ++k) dst[sample_lo<EX, X2>(own_pos<EX>(c.r, c.t, k), 0)] = acc[k];
+};
+
+// Inverse rows. Without COPY a block holds its tiles for the fields of one group and reads bins straight
+// from the workspace; with it two tiles share a TileFeed.
+template <class EX, bool X2, int KIND, uint32_t MF, bool COPY>
+__global__ void __launch_bounds__(RowBlock<EX, COPY ? 2 : row_tiles<EX>()>::THREADS, RowBlock<EX, COPY ? 2 : row_tiles<EX>()>::MINB)
+    k_rows_inv(const __grid_constant__ PassParams p, const __grid_constant__ TileMap map) {
+  constexpr int T = COPY ? 2 : row_tiles<EX>();
+  using SH = RowBlock<EX, T>;
+  constexpr int E = EX::E, H = E / 2;
+  static_assert(!COPY || KIND != EPI_OVERLAP, "the overlap sums are taken by whole blocks");
+  TOP_DYN_SMEM(float2, smem);
+  const RowLane<EX, T> c(smem);
+  RowEpilogue<EX, X2, KIND> epi;
+  float2 v[E];
+  float2 lo[H], hi[H];
+  if constexpr (COPY) {
+    TileFeed<EX> feed(smem, p.ny, p.nfields, p.group, p.l2_ahead);
+    if (threadIdx.x == 0) feed.start(map);
+#pragma unroll 1
+    while (feed.take(map, c, p.fault, v)) {
+      EX::template inv_from<false>(v, c.qbuf(), c.qt(), [] {}, c.buf(), c.t(), [&] { c.quad_sync(); }, p.twx);
+      if (c.r()) unfold_odd<EX, X2>(v, p.wpx, c.t());
+      trade_combine<EX, X2>(v, lo, hi, c.buf(), c.peer(), c.r(), c.t(), [] { EX::sync_group(); }, [&] { c.pair_sync(); });
+      const int f = feed.field(), g = feed.item() / feed.ntiles, y = feed.y0() + c.row();
+      const bool first = f == g * p.group;
+      if (first) epi.open(p, c, g, y);
+      epi.template field<MF>(p, c, f, g, first, y, lo, hi);
+      if (f + 1 == feed.end_field(feed.item())) epi.close(p, c, g, y);
     }
+  } else {
+    const int tile0 = (blockIdx.x * SH::T + c.tile()) * SH::ROWS;
+    const int y = tile0 + c.row();
+    const int g = blockIdx.y;
+    const int f0 = g * p.group, f1 = min(f0 + p.group, p.nfields);
+    epi.open(p, c, g, y);
+#pragma unroll 1
+    for (int f = f0; f < f1; ++f) {
+      load_bins<EX>(p, f, c, tile0 + c.qrow(), v);
+      EX::template inv_from<true>(
+          v, c.qbuf(), c.qt(),
+          [&] {
+            if (f > f0) c.tile_sync();  // the previous field's trade has been read
+          },
+          c.buf(), c.t(), [&] { c.quad_sync(); }, p.twx);
+      if (c.r()) unfold_odd<EX, X2>(v, p.wpx, c.t());
+      trade_combine<EX, X2>(v, lo, hi, c.buf(), c.peer(), c.r(), c.t(), [] { EX::sync_group(); }, [&] { c.pair_sync(); });
+      epi.template field<MF>(p, c, f, g, f == f0, y, lo, hi);
+      if constexpr (KIND == EPI_OVERLAP) {
+        // the block's sums in a fixed order: every thread's three values, added by thread 0
+        __syncthreads();
+        double* red = reinterpret_cast<double*>(smem);
+        red[3 * threadIdx.x] = epi.ov.re;
+        red[3 * threadIdx.x + 1] = epi.ov.im;
+        red[3 * threadIdx.x + 2] = epi.ov.pw;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+          double sr = 0.0, si = 0.0, sp = 0.0;
+          for (int i = 0; i < SH::THREADS; ++i) {
+            sr += red[3 * i];
+            si += red[3 * i + 1];
+            sp += red[3 * i + 2];
+          }
+          double* o = p.ov_part + ((long long)f * gridDim.x + blockIdx.x) * 3;
+          o[0] = sr;
+          o[1] = si;
+          o[2] = sp;
+        }
+        __syncthreads();
+      }
+    }
+    epi.close(p, c, g, y);
   }
 }
 
@@ -854,54 +1202,76 @@ __global__ void __launch_bounds__(RowShape<EX>::THREADS, RowShape<EX>::MINB) k_r
 // The inverse row pass of one propagation (pa) fused with the forward row pass of the next (pb) in a
 // system chain (Eq. 1 and Eq. 4 in turn): the field between them stays in registers and reaches
 // global memory only when it is kept (pa.out). pb's bins replace pa's in the workspace, tile by tile,
-// each block reading its tile before writing it.
-template <class EX, bool X2, uint32_t MF>
-__global__ void __launch_bounds__(RowShape<EX>::THREADS, RowShape<EX>::MINB)
-    k_rows_chain(const __grid_constant__ PassParams pa, const __grid_constant__ PassParams pb) {
-  using SH = RowShape<EX>;
-  constexpr int E = EX::E, M = EX::M, H = E / 2;
+// each tile read before it is written. With COPY tiles come by TileFeed and leave by copy.
+template <class EX, bool X2, uint32_t MF, bool COPY>
+__global__ void __launch_bounds__(RowBlock<EX, COPY ? 2 : row_tiles<EX>()>::THREADS, RowBlock<EX, COPY ? 2 : row_tiles<EX>()>::MINB)
+    k_rows_chain(const __grid_constant__ PassParams pa, const __grid_constant__ PassParams pb,
+                 const __grid_constant__ TileMap map) {
+  constexpr int T = COPY ? 2 : row_tiles<EX>();
+  using SH = RowBlock<EX, T>;
+  constexpr int E = EX::E, H = E / 2;
   TOP_DYN_SMEM(float2, smem);
-  const RowLane<EX> c(smem);
-  const int tile0 = (blockIdx.x * SH::TILES + c.tile) * SH::ROWS;
-  const int y = tile0 + c.row;
-  const int f = blockIdx.y;
+  const RowLane<EX, T> c(smem);
   const int nx = pa.nx;
-  const bool live = y < pa.ny;
-  float2 v[E];
-  load_bins<EX>(pa, f, c, tile0 + c.qrow, v);
-  EX::template inv_from<true>(v, c.qbuf, c.qt, [] {}, c.buf, c.t, [&] { c.quad_sync(); }, pa.twx);
-  if (c.r) unfold_odd<EX, X2>(v, pa.wpx, c.t);
-  float2 lo[H], hi[H];
-  trade_combine<EX, X2>(v, lo, hi, c.buf, c.peer, c.r, c.t, [] { EX::sync_group(); }, [&] { c.pair_sync(); });
   const ModDev& m = pb.msrc;
   const uint32_t flags = mod_flags<MF>(m);
-  const FieldSet& fsb = pb.sets[pb.set_of[f]];
-  const ModRow mr = mod_row(m, flags, fsb.src_lx, fsb.src_ly, f, live ? y : 0, nx);
-  float2* kept = pa.out ? pa.out + (long long)f * pa.out_stride + (long long)y * nx : nullptr;
-  const int n = live ? nx : 0;
-  auto samples = [&](float2 (&val)[H], bool hi_part) {
-    const OwnSamples<EX, X2> at{c.r, c.t, pa.ox, hi_part};
-    if (kept) {
+  float2 v[E];
+  // bins of (f, rows from tile0) in v to the next propagation's bins in v
+  auto tile = [&](int f, int tile0) {
+    const int y = tile0 + c.row();
+    const bool live = y < pa.ny;
+    EX::template inv_from<!COPY>(
+        v, c.qbuf(), c.qt(),
+        [&] {
+          if constexpr (COPY) copy_out_done(c);
+        },
+        c.buf(), c.t(), [&] { c.quad_sync(); }, pa.twx);
+    if (c.r()) unfold_odd<EX, X2>(v, pa.wpx, c.t());
+    float2 lo[H], hi[H];
+    trade_combine<EX, X2>(v, lo, hi, c.buf(), c.peer(), c.r(), c.t(), [] { EX::sync_group(); }, [&] { c.pair_sync(); });
+    const FieldSet& fsb = pb.sets[pb.set_of[f]];
+    const ModRow mr = mod_row(m, flags, fsb.src_lx, fsb.src_ly, f, live ? y : 0, nx);
+    float2* kept = pa.out ? pa.out + (long long)f * pa.out_stride + (long long)y * nx : nullptr;
+    const int n = live ? nx : 0;
+    auto samples = [&](float2 (&val)[H], bool hi_part) {
+      const OwnSamples<EX, X2> at{c.r(), c.t(), pa.ox, hi_part};
+      if (kept) {
+#pragma unroll
+        for (int k = 0; k < H; ++k)
+          if ((unsigned)at(k) < (unsigned)n) kept[at(k)] = val[k];
+      }
+      if (MF != 0) {
+        float2 mv[H];
+        mod_values(m, flags, m.conj, mr, nx, at, mv);
+#pragma unroll
+        for (int k = 0; k < H; ++k) val[k] = c_mul(val[k], mv[k]);
+      }
 #pragma unroll
       for (int k = 0; k < H; ++k)
-        if ((unsigned)at(k) < (unsigned)n) kept[at(k)] = val[k];
-    }
-    if (MF != 0) {
-      float2 mv[H];
-      mod_values(m, flags, m.conj, mr, nx, at, mv);
-#pragma unroll
-      for (int k = 0; k < H; ++k) val[k] = c_mul(val[k], mv[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < H; ++k)
-      if ((unsigned)at(k) >= (unsigned)n) val[k] = make_float2(0.f, 0.f);
+        if ((unsigned)at(k) >= (unsigned)n) val[k] = make_float2(0.f, 0.f);
+    };
+    samples(lo, false);
+    if constexpr (!X2) samples(hi, true);
+    trade_fold<EX, X2>(v, lo, hi, c.buf(), c.peer(), c.r(), c.t(), [&] { c.pair_sync(); });
+    if (c.r()) fold_odd<EX, X2>(v, pb.wpx, c.t());
+    EX::template fwd_to<true>(v, c.buf(), c.t(), pb.twx, [&] { c.pair_sync(); }, c.qbuf(), c.qt(), [&] { c.quad_sync(); });
   };
-  samples(lo, false);
-  if constexpr (!X2) samples(hi, true);
-  trade_fold<EX, X2>(v, lo, hi, c.buf, c.peer, c.r, c.t, [&] { c.pair_sync(); });
-  if (c.r) fold_odd<EX, X2>(v, pb.wpx, c.t);
-  EX::template fwd_to<true>(v, c.buf, c.t, pb.twx, [&] { c.pair_sync(); }, c.qbuf, c.qt, [&] { c.quad_sync(); });
-  store_bins<EX>(pb, f, c, tile0 + c.qrow, v);
+  if constexpr (COPY) {
+    TileFeed<EX> feed(smem, pa.ny, pa.nfields, 1, pa.l2_ahead);
+    if (threadIdx.x == 0) feed.start(map);
+#pragma unroll 1
+    while (feed.take(map, c, pa.fault, v)) {
+      tile(feed.field(), feed.y0());
+      copy_bins_out<EX>(map, feed.field(), c, feed.y0(), v);
+    }
+    if (c.hlead()) top_bulk_wait();
+  } else {
+    const int tile0 = (blockIdx.x * SH::T + c.tile()) * SH::ROWS;
+    const int f = blockIdx.y;
+    load_bins<EX>(pa, f, c, tile0 + c.qrow(), v);
+    tile(f, tile0);
+    store_bins<EX>(pb, f, c, tile0 + c.qrow(), v);
+  }
 }
 
 // ----------------------------------------------------------------------------- launchers
@@ -928,28 +1298,60 @@ constexpr uint32_t kPhase = TOP_MOD_PHASE;
 constexpr uint32_t kLensCirc = TOP_MOD_LENS | TOP_MOD_CIRC;
 constexpr uint32_t kPhaseCirc = TOP_MOD_PHASE | TOP_MOD_CIRC;
 
-template <class EX, bool X2, uint32_t MF>
-cudaError_t launch_rows_fwd_k(const PassParams& p, cudaStream_t s) {
+// Whether lines start on 16-byte boundaries, as tile copies need.
+template <class EX>
+inline bool copies(const PassParams& p) {
   using SH = RowShape<EX>;
-  static const cudaError_t attr = set_smem(k_rows_fwd<EX, X2, MF>, SH::SMEM);
+  return SH::COPY && (p.ny * SH::CI) % 2 == 0;
+}
+// The passes that also load tiles by copy want three tiles or more for each resident group of a launch:
+// one tile each, the pipeline only adds its start (one 1024 x 1024 field: inverse rows 13.5 us direct,
+// 14.7 by copy; four fields: 35.1 and 31.2; 16 fields at 512: 27.4 and 26.9).
+template <class EX>
+inline bool copies_in(const PassParams& p, int resident) {
+  return copies<EX>(p) && (long long)p.ny * p.nfields >= 6LL * RowShape<EX>::ROWS * resident;
+}
+template <class EX>
+inline cudaError_t tile_map(const PassParams& p, TileMap* map) {
+  using SH = RowShape<EX>;
+  return encode_tile_map(map, p.ws, p.ny * SH::CI, p.Px / SH::CI, p.nfields, p.ws_stride, SH::LB);
+}
+
+template <class EX, bool X2, uint32_t MF, bool COPY>
+cudaError_t launch_rows_fwd_k(const PassParams& p, cudaStream_t s) {
+  using SH = RowBlock<EX, row_tiles<EX>()>;
+  static const cudaError_t attr = set_smem(k_rows_fwd<EX, X2, MF, COPY>, SH::SMEM_X);
   if (attr != cudaSuccess) return attr;
-  static const int resident = resident_blocks(k_rows_fwd<EX, X2, MF>, SH::THREADS, SH::SMEM);
+  static const int resident = resident_blocks(k_rows_fwd<EX, X2, MF, COPY>, SH::THREADS, SH::SMEM_X);
   PassParams q = p;
   // bulk prefetches move whole 16-byte units
   q.l2_ahead = p.nx % 2 == 0 && !(p.tune_rows & TOP_TUNE_NO_L2_FWD) ? resident : 0;
-  dim3 grid((p.ny + SH::BLOCK_ROWS - 1) / SH::BLOCK_ROWS, p.nfields);
-  TOP_LAUNCH((k_rows_fwd<EX, X2, MF>), grid, SH::THREADS, SH::SMEM, s, q);
+  const int tiles = (p.ny + SH::BLOCK_ROWS - 1) / SH::BLOCK_ROWS;
+  const dim3 grid(COPY ? tiles * p.nfields : tiles, COPY ? 1 : p.nfields);
+  TileMap map{};
+  if (COPY) {
+    const cudaError_t e = tile_map<EX>(p, &map);
+    if (e != cudaSuccess) return e;
+  }
+  TOP_LAUNCH((k_rows_fwd<EX, X2, MF, COPY>), grid, SH::THREADS, SH::SMEM_X, s, q, map);
   return cudaGetLastError();
+}
+template <class EX, bool X2, uint32_t MF>
+cudaError_t launch_rows_fwd_m(const PassParams& p, cudaStream_t s) {
+  if constexpr (RowShape<EX>::COPY) {
+    if (copies<EX>(p)) return launch_rows_fwd_k<EX, X2, MF, true>(p, s);
+  }
+  return launch_rows_fwd_k<EX, X2, MF, false>(p, s);
 }
 
 template <class EX, bool X2>
 cudaError_t launch_rows_fwd_t(const PassParams& p, cudaStream_t s) {
   const uint32_t fl = p.msrc.flags;
-  if (fl == 0) return launch_rows_fwd_k<EX, X2, 0>(p, s);
+  if (fl == 0) return launch_rows_fwd_m<EX, X2, 0>(p, s);
   if constexpr (X2) {
-    if (fl == kPhase) return launch_rows_fwd_k<EX, X2, kPhase>(p, s);
+    if (fl == kPhase) return launch_rows_fwd_m<EX, X2, kPhase>(p, s);
   }
-  return launch_rows_fwd_k<EX, X2, TOP_MOD_DYNAMIC>(p, s);
+  return launch_rows_fwd_m<EX, X2, TOP_MOD_DYNAMIC>(p, s);
 }
 
 template <class EY, bool X2, int CI>
@@ -967,13 +1369,29 @@ cudaError_t launch_cols_k(const PassParams& p, cudaStream_t s) {
 
 template <class EX, bool X2, int KIND, uint32_t MF>
 cudaError_t launch_rows_inv_k(const PassParams& p, cudaStream_t s) {
-  using SH = RowShape<EX>;
-  static const cudaError_t attr = set_smem(k_rows_inv<EX, X2, KIND, MF>, SH::SMEM);
-  if (attr != cudaSuccess) return attr;
   PassParams q = p;
-  if (KIND == EPI_FIELD) q.group = 1;  // no sums: one field per block
-  dim3 grid((q.ny + SH::BLOCK_ROWS - 1) / SH::BLOCK_ROWS, (q.nfields + q.group - 1) / q.group);
-  TOP_LAUNCH((k_rows_inv<EX, X2, KIND, MF>), grid, SH::THREADS, SH::SMEM, s, q);
+  if (KIND == EPI_FIELD) q.group = 1;  // no sums: one field at a time
+  const int groups = (q.nfields + q.group - 1) / q.group;
+  if constexpr (RowShape<EX>::COPY && KIND != EPI_OVERLAP) {
+    using SH = RowBlock<EX, 2>;
+    static const cudaError_t attr = set_smem(k_rows_inv<EX, X2, KIND, MF, true>, SH::SMEM_DUO);
+    if (attr != cudaSuccess) return attr;
+    static const int resident = resident_blocks(k_rows_inv<EX, X2, KIND, MF, true>, SH::THREADS, SH::SMEM_DUO);
+    if (copies_in<EX>(p, resident)) {
+      TileMap map{};
+      const cudaError_t e = tile_map<EX>(p, &map);
+      if (e != cudaSuccess) return e;
+      const int items = (p.ny + SH::ROWS - 1) / SH::ROWS * groups;
+      q.l2_ahead = 2 * resident;  // both groups of every resident block
+      TOP_LAUNCH((k_rows_inv<EX, X2, KIND, MF, true>), items, SH::THREADS, SH::SMEM_DUO, s, q, map);
+      return cudaGetLastError();
+    }
+  }
+  using SH = RowBlock<EX, row_tiles<EX>()>;
+  static const cudaError_t attr = set_smem(k_rows_inv<EX, X2, KIND, MF, false>, SH::SMEM_X);
+  if (attr != cudaSuccess) return attr;
+  dim3 grid((q.ny + SH::BLOCK_ROWS - 1) / SH::BLOCK_ROWS, groups);
+  TOP_LAUNCH((k_rows_inv<EX, X2, KIND, MF, false>), grid, SH::THREADS, SH::SMEM_X, s, q, TileMap{});
   return cudaGetLastError();
 }
 
@@ -999,11 +1417,27 @@ cudaError_t launch_rows_inv_t(const PassParams& p, cudaStream_t s) {
 
 template <class EX, bool X2, uint32_t MF>
 cudaError_t launch_rows_chain_k(const PassParams& pa, const PassParams& pb, cudaStream_t s) {
-  using SH = RowShape<EX>;
-  static const cudaError_t attr = set_smem(k_rows_chain<EX, X2, MF>, SH::SMEM);
+  if constexpr (RowShape<EX>::COPY) {
+    using SH = RowBlock<EX, 2>;
+    static const cudaError_t attr = set_smem(k_rows_chain<EX, X2, MF, true>, SH::SMEM_DUO);
+    if (attr != cudaSuccess) return attr;
+    static const int resident = resident_blocks(k_rows_chain<EX, X2, MF, true>, SH::THREADS, SH::SMEM_DUO);
+    if (copies_in<EX>(pa, resident)) {
+      TileMap map{};
+      const cudaError_t e = tile_map<EX>(pa, &map);
+      if (e != cudaSuccess) return e;
+      const int items = (pa.ny + SH::ROWS - 1) / SH::ROWS * pa.nfields;
+      PassParams qa = pa;
+      qa.l2_ahead = 0;  // its tiles are a while in coming; prefetches measured slower (9.7 -> 10.0 us a field)
+      TOP_LAUNCH((k_rows_chain<EX, X2, MF, true>), items, SH::THREADS, SH::SMEM_DUO, s, qa, pb, map);
+      return cudaGetLastError();
+    }
+  }
+  using SH = RowBlock<EX, row_tiles<EX>()>;
+  static const cudaError_t attr = set_smem(k_rows_chain<EX, X2, MF, false>, SH::SMEM_X);
   if (attr != cudaSuccess) return attr;
   dim3 grid((pa.ny + SH::BLOCK_ROWS - 1) / SH::BLOCK_ROWS, pa.nfields);
-  TOP_LAUNCH((k_rows_chain<EX, X2, MF>), grid, SH::THREADS, SH::SMEM, s, pa, pb);
+  TOP_LAUNCH((k_rows_chain<EX, X2, MF, false>), grid, SH::THREADS, SH::SMEM_X, s, pa, pb, TileMap{});
   return cudaGetLastError();
 }
 

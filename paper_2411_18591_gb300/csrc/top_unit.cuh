@@ -14,7 +14,7 @@ inline void fill_engine_info(EngineInfo* info) {
   info->NS = EN::NS;
   for (int s = 0; s < 4; ++s) info->R[s] = s < EN::NS ? EN::radix(s) : 1;
   info->tw_size = EN::TW_SIZE;
-  info->rows = RowShape<EN>::BLOCK_ROWS;
+  info->rows = RowShape<EN>::ROWS * row_tiles<EN>();
   info->ci = RowShape<EN>::CI;
 }
 

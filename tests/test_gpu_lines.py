@@ -75,3 +75,32 @@ def test_tile_edges(T, ny, nx, pad):
     assert torch.equal(keep, first)
     assert torch.equal(y, T.top_propagate(first, dy, dx, lams, 0.5 * z, pad, pre=pre))
     assert rel_l2(host(inten), (np.abs(host(y).astype(np.complex128)) ** 2).sum(0)) < TOL
+
+
+# batches large enough for the row passes to move their tiles by copy, at every plan that does: whole and
+# part-filled last tiles, one-field and grouped items, groups of different lengths
+@pytest.mark.parametrize("ny,nx,batch", [(16, 256, 800), (250, 256, 48), (250, 512, 32), (16, 768, 256), (16, 1000, 160),
+                                         (16, 1024, 264), (250, 1024, 16), (16, 2048, 128)])
+def test_copied_tiles_match_direct_ones(T, ny, nx, batch):
+    d, z, lam = 6e-6, 0.02, 600e-9
+    gen = torch.Generator(device="cuda").manual_seed(ny * 3 + nx)
+    x = torch.randn((batch, ny, nx), generator=gen, device="cuda", dtype=torch.complex64)
+    phi = torch.rand((ny, nx), generator=gen, device="cuda") * 6 - 3
+    pre = T.Modulation(phase=phi)
+    stages = [T.Stage(z, pre=pre), T.Stage(0.5 * z, pre=T.Modulation(focal_length=0.3, radius=0.4 * nx * d))]
+    out = T.top_propagate(x, d, d, lam, z, 2.0, pre=pre)
+    group = 4
+    y, inten = T.top_fused_chain(x, d, d, lam, stages, 2.0, intensity_group=group)
+    gp, direct = torch.zeros_like(phi), torch.zeros(ny, nx, dtype=torch.float64, device="cuda")
+    back = T.top_propagate_backward(x, d, d, lam, z, 2.0, pre=pre, saved_in=out, grad_phase=gp)
+    for b in range(batch):
+        assert torch.equal(out[b], T.top_propagate(x[b], d, d, lam, z, 2.0, pre=pre)[0]), b
+        y1, i1 = T.top_fused_chain(x[b], d, d, lam, stages, 2.0, intensity_group=1)
+        assert torch.equal(y[b], y1[0]), b
+        g1 = torch.zeros_like(phi)
+        assert torch.equal(back[b], T.top_propagate_backward(x[b], d, d, lam, z, 2.0, pre=pre, saved_in=out[b],
+                                                             grad_phase=g1)), b
+        direct += g1
+    ref = (y.abs().double() ** 2).reshape(batch // group, group, ny, nx).sum(1)
+    assert rel_l2(host(inten), host(ref)) < TOL
+    assert rel_l2(host(gp), host(direct)) < TOL
