@@ -945,8 +945,8 @@ top_status bluestein_fields(top_handle h, const Request& q, const Geometry& geo,
       fin = src;
       in_rep = 1;
     }
-    TOP_CUDA(cudaMemcpyAsync(d_h, tables.data() + pos, size_t(n) * sizeof(void*), cudaMemcpyHostToDevice, st),
-             "cudaMemcpyAsync(transfer table pointers)");
+    // by kernels that carry the pointers in their parameters: a copy from pageable memory waits for the stream
+    TOP_CUDA(launch_put(d_h, tables.data() + pos, size_t(n) * sizeof(void*), st), "transfer table pointers");
     CztParams r{};
     r.mode = CZT_FWD;
     r.in = fin;
