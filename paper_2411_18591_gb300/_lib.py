@@ -131,6 +131,9 @@ def check(status: int) -> None:
         raise TopError(status, msg)
 
 
+_OneDouble = C.c_double * 1
+
+
 def doubles(values) -> C.Array:
     vals = [float(v) for v in values]
-    return (C.c_double * len(vals))(*vals)
+    return (_OneDouble if len(vals) == 1 else C.c_double * len(vals))(*vals)

@@ -28,9 +28,15 @@ _handle_lock = threading.Lock()
 
 def handle(device: Optional[torch.device] = None) -> C.c_void_p:
     """The library handle of a CUDA device (created on first use, kept for the process)."""
+    idx = None
+    if device is not None:
+        idx = (device if isinstance(device, torch.device) else torch.device(device)).index
+    if idx is None:
+        idx = torch.cuda.current_device()
+    h = _handles.get(idx)
+    if h is not None:
+        return h
     lib = _lib.load()
-    dev = torch.device("cuda", torch.cuda.current_device()) if device is None else torch.device(device)
-    idx = dev.index if dev.index is not None else torch.cuda.current_device()
     with _handle_lock:
         h = _handles.get(idx)
         if h is None:
@@ -41,7 +47,11 @@ def handle(device: Optional[torch.device] = None) -> C.c_void_p:
 
 
 def _stream(t: torch.Tensor) -> C.c_void_p:
-    return C.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
+    # the raw handle of torch's current stream: a Stream object costs small calls more than the rest of
+    # their arguments
+    if not t.is_cuda:
+        raise ValueError(f"expected a cuda tensor, got one on {t.device}")
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(t.get_device()))
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
