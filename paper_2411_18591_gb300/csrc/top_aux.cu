@@ -555,7 +555,7 @@ cudaError_t launch_resample(const float2* in, float2* out, long long batch, Resa
 }
 
 cudaError_t encode_tile_map(TileMap* map, const void* ws, long long samples, long long lines, int nfields,
-                            long long field_stride, int box_lines) {
+                            long long field_stride, int box_lines, bool with_wide) {
   using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                               const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -570,6 +570,7 @@ cudaError_t encode_tile_map(TileMap* map, const void* ws, long long samples, lon
   const cuuint64_t strides[2] = {cuuint64_t(samples) * sizeof(float2), cuuint64_t(field_stride) * sizeof(float2)};
   const cuuint32_t step[3] = {1, 1, 1};
   for (const bool wide : {false, true}) {
+    if (wide && !with_wide) break;
     const cuuint32_t box[3] = {wide ? 16u : 4u, cuuint32_t(box_lines), 1};
     // a sample is moved as one 8-byte element
     const CUresult r = encode(wide ? &map->wide : &map->tile, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, const_cast<void*>(ws),

@@ -170,7 +170,7 @@ struct TileMap {
   CUtensorMap wide;
 };
 cudaError_t encode_tile_map(TileMap* map, const void* ws, long long samples, long long lines, int nfields,
-                            long long field_stride, int box_lines);
+                            long long field_stride, int box_lines, bool with_wide);
 
 // The autotune table (top_tune.cu): TOP_TUNE_* flags per line length M (0: the defaults).
 uint32_t tune_flags(int M);

@@ -1312,9 +1312,9 @@ inline bool copies_in(const PassParams& p, int resident) {
   return copies<EX>(p) && (long long)p.ny * p.nfields >= 6LL * RowShape<EX>::ROWS * resident;
 }
 template <class EX>
-inline cudaError_t tile_map(const PassParams& p, TileMap* map) {
+inline cudaError_t tile_map(const PassParams& p, TileMap* map, bool with_wide) {
   using SH = RowShape<EX>;
-  return encode_tile_map(map, p.ws, p.ny * SH::CI, p.Px / SH::CI, p.nfields, p.ws_stride, SH::LB);
+  return encode_tile_map(map, p.ws, p.ny * SH::CI, p.Px / SH::CI, p.nfields, p.ws_stride, SH::LB, with_wide);
 }
 
 template <class EX, bool X2, uint32_t MF, bool COPY>
@@ -1330,7 +1330,7 @@ cudaError_t launch_rows_fwd_k(const PassParams& p, cudaStream_t s) {
   const dim3 grid(COPY ? tiles * p.nfields : tiles, COPY ? 1 : p.nfields);
   TileMap map{};
   if (COPY) {
-    const cudaError_t e = tile_map<EX>(p, &map);
+    const cudaError_t e = tile_map<EX>(p, &map, false);
     if (e != cudaSuccess) return e;
   }
   TOP_LAUNCH((k_rows_fwd<EX, X2, MF, COPY>), grid, SH::THREADS, SH::SMEM_X, s, q, map);
@@ -1379,7 +1379,7 @@ cudaError_t launch_rows_inv_k(const PassParams& p, cudaStream_t s) {
     static const int resident = resident_blocks(k_rows_inv<EX, X2, KIND, MF, true>, SH::THREADS, SH::SMEM_DUO);
     if (copies_in<EX>(p, resident)) {
       TileMap map{};
-      const cudaError_t e = tile_map<EX>(p, &map);
+      const cudaError_t e = tile_map<EX>(p, &map, true);
       if (e != cudaSuccess) return e;
       const int items = (p.ny + SH::ROWS - 1) / SH::ROWS * groups;
       q.l2_ahead = 2 * resident;  // both groups of every resident block
@@ -1424,7 +1424,7 @@ cudaError_t launch_rows_chain_k(const PassParams& pa, const PassParams& pb, cuda
     static const int resident = resident_blocks(k_rows_chain<EX, X2, MF, true>, SH::THREADS, SH::SMEM_DUO);
     if (copies_in<EX>(pa, resident)) {
       TileMap map{};
-      const cudaError_t e = tile_map<EX>(pa, &map);
+      const cudaError_t e = tile_map<EX>(pa, &map, false);
       if (e != cudaSuccess) return e;
       const int items = (pa.ny + SH::ROWS - 1) / SH::ROWS * pa.nfields;
       PassParams qa = pa;
