@@ -2457,9 +2457,20 @@ static top_status coh_check(const top_grid* g, const double* lambda, const doubl
   return TOP_OK;
 }
 
-// P or P^H applied over r2 (each r1 slice), then over r1 via two batched transposes (Eq. 13).
+// The scratch of a coherence call: a tensor for the transposed halves and, behind it, coh_work bytes. Every
+// call asks for both, so that one warm call allocates for all of them.
+static top_status coh_buffers(top_handle h, const top_grid* g, void** t, float2** work) {
+  const size_t n = size_t(g->ny) * g->nx;
+  const size_t tensor = (sizeof(float2) * size_t(g->batch) * n * n + 255) / 256 * 256;
+  TOP_TRY(coh_scratch(h, tensor + coh_work(int(n)), t));
+  *work = reinterpret_cast<float2*>(static_cast<char*>(*t) + tensor);
+  return TOP_OK;
+}
+
+// P or P^H applied over r2 (each r1 slice), then over r1 via a batched transpose (Eq. 13) into t; the
+// result stays transposed there. dst holds the first half's result.
 static top_status coh_two_sided(top_handle h, const top_grid* g, const void* src, void* dst, const double* lambda,
-                                const double* z, int adjoint_r2, cudaStream_t st) {
+                                const double* z, int adjoint_r2, void* t, cudaStream_t st) {
   const int n = g->ny * g->nx;
   top_grid fg = *g;
   fg.batch = g->batch * n;
@@ -2468,15 +2479,16 @@ static top_status coh_two_sided(top_handle h, const top_grid* g, const void* src
   q.src_kind = SRC_FIELD; q.in = src; q.group = 1;
   q.epi_kind = EPI_FIELD; q.out = dst;
   TOP_TRY(run_propagation(h, q, st));
-  void* tmp = nullptr;
-  TOP_TRY(coh_scratch(h, sizeof(float2) * size_t(g->batch) * n * n, &tmp));
   TOP_TRY(timed(h, KK_AUX, st, "transpose", [&] {
-    return launch_transpose(static_cast<const float2*>(dst), static_cast<float2*>(tmp), g->batch, n, st);
+    return launch_transpose(static_cast<const float2*>(dst), static_cast<float2*>(t), g->batch, n, st);
   }));
-  q.in = tmp; q.out = tmp; q.adjoint = 1 - adjoint_r2;
-  TOP_TRY(run_propagation(h, q, st));
+  q.in = t; q.out = t; q.adjoint = 1 - adjoint_r2;
+  return run_propagation(h, q, st);
+}
+// ... and back to [r1][r2] in dst.
+static top_status coh_untranspose(top_handle h, const top_grid* g, const void* t, void* dst, cudaStream_t st) {
   return timed(h, KK_AUX, st, "transpose", [&] {
-    return launch_transpose(static_cast<const float2*>(tmp), static_cast<float2*>(dst), g->batch, n, st);
+    return launch_transpose(static_cast<const float2*>(t), static_cast<float2*>(dst), g->batch, g->ny * g->nx, st);
   });
 }
 
@@ -2490,16 +2502,21 @@ top_status top_propagate_coherence(top_handle h, const top_grid* g, const void* 
   TOP_TRY(bind(h));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const void* src = gamma_in;
+  void* t = nullptr;
+  float2* work = nullptr;
+  TOP_TRY(coh_buffers(h, g, &t, &work));
   if (mask && mask->flags) {
     PassParams mp;
     TOP_TRY(coh_mask_params(h, g, mask, lambda[0], &mp));
     TOP_TRY(timed(h, KK_AUX, st, "coherence modulation", [&] {
-      return launch_coh_modulate(static_cast<const float2*>(gamma_in), static_cast<float2*>(gamma_out), mp, g->batch, 0, st);
+      return launch_coh_modulate(static_cast<const float2*>(gamma_in), static_cast<float2*>(gamma_out), mp, g->batch,
+                                 work, st);
     }));
     src = gamma_out;
   }
   // Gamma_z = P Gamma P^H: conj(H) over (y2, x2), H over (y1, x1)
-  return coh_two_sided(h, g, src, gamma_out, lambda, z, 1, st);
+  TOP_TRY(coh_two_sided(h, g, src, gamma_out, lambda, z, 1, t, st));
+  return coh_untranspose(h, g, t, gamma_out, st);
 }
 
 top_status top_propagate_coherence_backward(top_handle h, const top_grid* g, const void* grad_out, void* grad_in,
@@ -2523,35 +2540,26 @@ top_status top_propagate_coherence_backward(top_handle h, const top_grid* g, con
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int n = g->ny * g->nx;
   const size_t tensor = sizeof(float2) * size_t(g->batch) * n * n;
-  // G' = P^H G P lands in grad_in, or (when the caller wants no grad_in) in a scratch tensor the
-  // handle keeps: the two-sided propagation uses the workspace and the transpose scratch already
+  // the first half of G' = P^H G P goes through grad_in, or (when the caller wants no grad_in) through a
+  // scratch tensor the handle keeps: the two-sided propagation uses the workspace and the transpose scratch
   void* dst = grad_in;
   if (!dst) {
     TOP_TRY(grow_scratch(&h->cohg, &h->cohg_bytes, tensor, "cudaMalloc(coherence gradient)"));
     dst = h->cohg;
   }
-  top_status s = coh_two_sided(h, g, grad_out, dst, lambda, z, 0, st);
-  if (s == TOP_OK && pg) {
-    PassParams mp;
-    s = coh_mask_params(h, g, mask, lambda[0], &mp);
-    const size_t work = coh_mask_grads_work(int(n)) + 256;
-    if (s == TOP_OK && h->ws_bytes < work) s = ensure_workspace(h, work);
-    if (s == TOP_OK)
-      s = timed(h, KK_AUX, st, "coherence mask gradients", [&] {
-        return launch_coh_mask_grads(static_cast<const float2*>(dst), static_cast<const float2*>(grads->saved_in), mp,
-                                     g->batch, static_cast<float2*>(h->ws), grads->grad_phase, grads->grad_amplitude,
-                                     static_cast<float2*>(grads->grad_mask), st);
-      });
-  }
-  if (s == TOP_OK && grad_in && mask && mask->flags) {
-    PassParams mp;
-    s = coh_mask_params(h, g, mask, lambda[0], &mp);
-    if (s == TOP_OK)
-      s = timed(h, KK_AUX, st, "coherence modulation backward", [&] {
-        return launch_coh_modulate(static_cast<const float2*>(dst), static_cast<float2*>(dst), mp, g->batch, 1, st);
-      });
-  }
-  return s;
+  void* t = nullptr;
+  float2* work = nullptr;
+  TOP_TRY(coh_buffers(h, g, &t, &work));
+  TOP_TRY(coh_two_sided(h, g, grad_out, dst, lambda, z, 0, t, st));
+  if (!mask || !mask->flags) return coh_untranspose(h, g, t, grad_in, st);
+  PassParams mp;
+  TOP_TRY(coh_mask_params(h, g, mask, lambda[0], &mp));
+  return timed(h, KK_AUX, st, "coherence backward", [&] {
+    return launch_coh_backward_end(static_cast<const float2*>(t), pg ? static_cast<const float2*>(grads->saved_in) : nullptr,
+                                   mp, g->batch, work, static_cast<float2*>(grad_in),
+                                   pg ? grads->grad_phase : nullptr, pg ? grads->grad_amplitude : nullptr,
+                                   pg ? static_cast<float2*>(grads->grad_mask) : nullptr, st);
+  });
 }
 
 static top_status intensity_check(top_handle h, const top_grid* g, const void* field, const void* other, int64_t group,

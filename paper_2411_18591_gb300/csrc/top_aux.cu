@@ -720,17 +720,21 @@ __device__ __forceinline__ float2 coh_mask(const PassParams& p, int r) {
   return mod_value(p.msrc, p.msrc.flags, 0, fs.src_lx, fs.src_ly, 0, y, x, p.nx);
 }
 
-// out(r1, r2) = M(r1) conj(M(r2)) in(r1, r2)  (Eq. 12), or its conjugate factor for the backward
-__global__ void __launch_bounds__(256) k_coh_modulate(const float2* in, float2* out, const __grid_constant__ PassParams p,
-                                                      int n, int conj_mask) {
+// M(s) for every s of the grid (the mask of Eq. 12, evaluated once)
+__global__ void __launch_bounds__(256) k_coh_mask_values(const __grid_constant__ PassParams p, int n, float2* mv) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s < n) mv[s] = coh_mask(p, s);
+}
+
+// out(r1, r2) = M(r1) conj(M(r2)) in(r1, r2)  (Eq. 12). From the mask's values mv (both factors worked out per element took 97 us on a 64^4 tensor; the two
+// reads and the write of it take 40 at the copy rate).
+__global__ void __launch_bounds__(256) k_coh_modulate(const float2* in, float2* out, const float2* mv, int n) {
   const int r2 = blockIdx.x * blockDim.x + threadIdx.x;
   const int r1 = blockIdx.y;
   const long long b = blockIdx.z;
   if (r2 >= n) return;
-  float2 d = c_mulc(coh_mask(p, r1), coh_mask(p, r2));
-  if (conj_mask) d = c_conj(d);
   const long long i = (b * n + r1) * n + r2;
-  out[i] = c_mul(in[i], d);
+  out[i] = c_mul(in[i], c_mulc(__ldg(mv + r1), __ldg(mv + r2)));
 }
 
 // batched square transpose through a 32 x 33 shared tile
@@ -761,68 +765,91 @@ __global__ void __launch_bounds__(256) k_coh_diag_backward(const float* gI, floa
   if (r < n) grad[(b * n + r) * n + r] = make_float2(gI[b * n + r], 0.f);
 }
 
-// M(s) for every s of the grid (the mask of Eq. 12, evaluated once for the gradient sums)
-__global__ void __launch_bounds__(256) k_coh_mask_values(const __grid_constant__ PassParams p, int n, float2* mv) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < n) mv[s] = coh_mask(p, s);
-}
-
-// row term: one block per r, fixed tree order over s; batch summed in order
-__global__ void __launch_bounds__(256) k_coh_grad_rows(const float2* G, const float2* Gm, const float2* mv, int n,
-                                                       long long batch, float2* gm) {
-  __shared__ float2 red[256];
-  const int r = blockIdx.x;
-  float2 acc = make_float2(0.f, 0.f);
-  for (long long b = 0; b < batch; ++b) {
-    const long long row = (b * n + r) * n;
-    for (int s = threadIdx.x; s < n; s += blockDim.x) acc = c_add(acc, c_mul(c_mulc(G[row + s], Gm[row + s]), mv[s]));
-  }
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int k = 128; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] = c_add(red[threadIdx.x], red[threadIdx.x + k]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) gm[r] = red[0];
-}
-
-// column term, partial sums: block (32 r, kCohWarps warps) of slice `split` of the s range; warp w
-// sums its part of the slice in order (over the batch, then s), and the warps' sums are added in
-// warp order: part[split][r]
-constexpr int kCohSplit = 16;
-constexpr int kCohWarps = 8;
-__global__ void __launch_bounds__(32 * kCohWarps) k_coh_grad_cols_part(const float2* G, const float2* Gm, const float2* mv,
-                                                                       int n, long long batch, float2* part) {
-  __shared__ float2 red[kCohWarps][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int r = blockIdx.x * 32 + lane;
-  const int per = (n + kCohSplit * kCohWarps - 1) / (kCohSplit * kCohWarps);
-  const int s0 = (blockIdx.y * kCohWarps + w) * per, s1 = min(n, s0 + per);
-  float2 acc = make_float2(0.f, 0.f);
-  if (r < n) {
-    for (long long b = 0; b < batch; ++b)
-      for (int s = s0; s < s1; ++s) {
-        const long long i = (b * n + s) * n + r;
-        acc = c_add(acc, c_mul(c_mulc(Gm[i], G[i]), mv[s]));
+// The end of the coherence backward in one pass over its two tensors: G' (transposed, Gt[r2][r1]) back to
+// [r1][r2], times conj(M(r1) conj(M(r2))) into out (if wanted), and, with the saved input Gm, the sums of
+// the mask gradient's row and column terms over the block's kCohRows x kCohCols samples (part_rows
+// [column block][r1], part_cols[row block][r2], each in a fixed order). Bound by HBM: 402 MB on a 64^4
+// tensor (two tensors read, one written), where the transpose, the two sums and the modulation as passes
+// of their own moved 1.2 GB (246 us).
+constexpr int kCohRows = 64, kCohCols = 128;
+__global__ void __launch_bounds__(256) k_coh_backward_end(const float2* Gt, const float2* Gm, const float2* mv, int n,
+                                                          long long batch, float2* out, float2* part_rows,
+                                                          float2* part_cols) {
+  __shared__ float2 tile[32][33];
+  __shared__ float2 red[8][32];
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int r0 = blockIdx.y * kCohRows, c0 = blockIdx.x * kCohCols;
+  float2 rows[kCohRows / 8];
+#pragma unroll
+  for (int k = 0; k < kCohRows / 8; ++k) rows[k] = make_float2(0.f, 0.f);
+#pragma unroll 1
+  for (int cb = 0; cb < kCohCols; cb += 32) {
+    const int col = c0 + cb + tx;
+    const float2 mc = col < n ? __ldg(mv + col) : make_float2(0.f, 0.f);
+    float2 cols = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (long long b = 0; b < batch; ++b) {
+      const long long base = b * n * n;
+#pragma unroll
+      for (int rb = 0; rb < kCohRows; rb += 32) {
+        float2 gm[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int c = c0 + cb + ty + 8 * k, r = r0 + rb + tx;
+          if (c < n && r < n) tile[ty + 8 * k][tx] = Gt[base + (long long)c * n + r];
+          const int row = r0 + rb + ty + 8 * k;
+          gm[k] = Gm && row < n && col < n ? Gm[base + (long long)row * n + col] : make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int row = r0 + rb + ty + 8 * k;
+          if (row < n && col < n) {
+            const float2 g = tile[tx][ty + 8 * k];
+            const float2 mr = __ldg(mv + row);
+            if (out) out[base + (long long)row * n + col] = c_mul(g, c_conj(c_mulc(mr, mc)));
+            if (Gm) {
+              rows[rb / 8 + k] = c_add(rows[rb / 8 + k], c_mul(c_mulc(g, gm[k]), mc));
+              cols = c_add(cols, c_mul(c_mulc(gm[k], g), mr));
+            }
+          }
+        }
+        __syncthreads();
       }
+    }
+    if (Gm) {
+      red[ty][tx] = cols;
+      __syncthreads();
+      if (ty == 0 && col < n) {
+        float2 t = red[0][tx];
+        for (int k = 1; k < 8; ++k) t = c_add(t, red[k][tx]);
+        part_cols[(long long)blockIdx.y * n + col] = t;
+      }
+      __syncthreads();
+    }
   }
-  red[w][lane] = acc;
-  __syncthreads();
-  if (w == 0 && r < n) {
-    float2 t = red[0][lane];
-    for (int k = 1; k < kCohWarps; ++k) t = c_add(t, red[k][lane]);
-    part[(long long)blockIdx.y * n + r] = t;
+  if (Gm) {
+#pragma unroll
+    for (int k = 0; k < kCohRows / 8; ++k) {
+      float2 t = rows[k];
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1)
+        t = c_add(t, make_float2(__shfl_xor_sync(0xffffffffu, t.x, d), __shfl_xor_sync(0xffffffffu, t.y, d)));
+      const int row = r0 + (k / 4) * 32 + ty + 8 * (k % 4);
+      if (tx == 0 && row < n) part_rows[(long long)blockIdx.x * n + row] = t;
+    }
   }
 }
 
-// g_M(r) = row term + the column slices in order; then the parameter gradients
+// g_M(r) = the row and column sums in order; then the parameter gradients
 __global__ void __launch_bounds__(256) k_coh_grad_finish(const __grid_constant__ PassParams p, int n,
-                                                         const float2* gm_rows, const float2* part, float* gphase,
-                                                         float* gamp, float2* gmask) {
+                                                         const float2* part_rows, int nrows, const float2* part_cols,
+                                                         int ncols, float* gphase, float* gamp, float2* gmask) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
-  float2 acc = gm_rows[r];
-  for (int k = 0; k < kCohSplit; ++k) acc = c_add(acc, part[(long long)k * n + r]);
+  float2 acc = make_float2(0.f, 0.f);
+  for (int k = 0; k < nrows; ++k) acc = c_add(acc, part_rows[(long long)k * n + r]);
+  for (int k = 0; k < ncols; ++k) acc = c_add(acc, part_cols[(long long)k * n + r]);
   // acc = g_M(r) for the complex mask value M(r)
   const int y = r / p.nx, x = r - (r / p.nx) * p.nx;
   const FieldSet& fs = p.sets[0];
@@ -839,13 +866,18 @@ __global__ void __launch_bounds__(256) k_coh_grad_finish(const __grid_constant__
   }
 }
 
-size_t coh_mask_grads_work(int n) { return sizeof(float2) * size_t(n) * (2 + kCohSplit); }
+size_t coh_work(int n) {
+  return sizeof(float2) * size_t(n) * (1 + (n + kCohCols - 1) / kCohCols + (n + kCohRows - 1) / kCohRows);
+}
 
-cudaError_t launch_coh_modulate(const float2* in, float2* out, const PassParams& p, long long batch, int conj_mask,
+cudaError_t launch_coh_modulate(const float2* in, float2* out, const PassParams& p, long long batch, float2* work,
                                 cudaStream_t s) {
   const int n = p.ny * p.nx;
+  TOP_LAUNCH(k_coh_mask_values, (n + 255) / 256, 256, 0, s, p, n, work);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   dim3 grid((n + 255) / 256, n, unsigned(batch));
-  TOP_LAUNCH(k_coh_modulate, grid, 256, 0, s, in, out, p, n, conj_mask);
+  TOP_LAUNCH(k_coh_modulate, grid, 256, 0, s, in, out, work, n);
   return cudaGetLastError();
 }
 
@@ -869,23 +901,22 @@ cudaError_t launch_coh_diag_backward(const float* gI, float2* grad, long long ba
   return cudaGetLastError();
 }
 
-cudaError_t launch_coh_mask_grads(const float2* G, const float2* gamma_in, const PassParams& p, long long batch,
-                                  float2* gm_work, float* grad_phase, float* grad_amp, float2* grad_mask,
-                                  cudaStream_t s) {
+cudaError_t launch_coh_backward_end(const float2* Gt, const float2* gamma_in, const PassParams& p, long long batch,
+                                    float2* work, float2* grad_in, float* grad_phase, float* grad_amp,
+                                    float2* grad_mask, cudaStream_t s) {
   const int n = p.ny * p.nx;
-  float2* rows = gm_work;
-  float2* mv = gm_work + n;
-  float2* part = gm_work + 2 * size_t(n);
+  const dim3 grid((n + kCohCols - 1) / kCohCols, (n + kCohRows - 1) / kCohRows);
+  float2* mv = work;
+  float2* rows = work + n;
+  float2* cols = rows + size_t(grid.x) * n;
   TOP_LAUNCH(k_coh_mask_values, (n + 255) / 256, 256, 0, s, p, n, mv);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  TOP_LAUNCH(k_coh_grad_rows, n, 256, 0, s, G, gamma_in, mv, n, batch, rows);
+  TOP_LAUNCH(k_coh_backward_end, grid, dim3(32, 8), 0, s, Gt, gamma_in, mv, n, batch, grad_in, rows, cols);
   e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  TOP_LAUNCH(k_coh_grad_cols_part, dim3((n + 31) / 32, kCohSplit), 32 * kCohWarps, 0, s, G, gamma_in, mv, n, batch, part);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  TOP_LAUNCH(k_coh_grad_finish, (n + 255) / 256, 256, 0, s, p, n, rows, part, grad_phase, grad_amp, grad_mask);
+  if (e != cudaSuccess || !gamma_in) return e;
+  TOP_LAUNCH(k_coh_grad_finish, (n + 255) / 256, 256, 0, s, p, n, rows, int(grid.x), cols, int(grid.y), grad_phase, grad_amp,
+             grad_mask);
   return cudaGetLastError();
 }
 

@@ -89,18 +89,19 @@ cudaError_t launch_transpose_rect(const float2* in, float2* out, long long batch
 namespace top {
 
 // Mutual coherence (Eq. 12-13), tensors [batch][n][n] with n = ny * nx.
-cudaError_t launch_coh_modulate(const float2* in, float2* out, const PassParams& p, long long batch, int conj_mask,
+// (work: the mask's values, ny nx samples)
+cudaError_t launch_coh_modulate(const float2* in, float2* out, const PassParams& p, long long batch, float2* work,
                                 cudaStream_t s);
 cudaError_t launch_transpose(const float2* in, float2* out, long long batch, int n, cudaStream_t s);
 cudaError_t launch_coh_diag(const float2* gamma, float* inten, long long batch, int n, cudaStream_t s);
 cudaError_t launch_coh_diag_backward(const float* gI, float2* grad, long long batch, int n, cudaStream_t s);
-// g_M(r) = sum_s G(r,s) conj(Gm(r,s)) M(s) + sum_s conj(G(s,r)) Gm(s,r) M(s), summed over the batch,
-// then turned into phase / amplitude / complex-mask gradients; gm_work holds
-// coh_mask_grads_work(ny nx) bytes (the row terms, the mask values and the column slices; the
-// column sum runs in slices over the grid, each slice in a fixed order, the slices in order).
-size_t coh_mask_grads_work(int n);
-cudaError_t launch_coh_mask_grads(const float2* G, const float2* gamma_in, const PassParams& p, long long batch,
-                                  float2* gm_work, float* grad_phase, float* grad_amp, float2* grad_mask,
-                                  cudaStream_t s);
+// The end of the backward, from G' transposed: grad_in = conj(M(r1) conj(M(r2))) G'(r1, r2) (optional) and,
+// with the saved input, the mask gradients of
+// g_M(r) = sum_s G(r,s) conj(Gm(r,s)) M(s) + sum_s conj(G(s,r)) Gm(s,r) M(s), summed over the batch in a
+// fixed order. work holds coh_work(ny nx) bytes (the mask's values and the blocks' partial sums).
+size_t coh_work(int n);
+cudaError_t launch_coh_backward_end(const float2* Gt, const float2* gamma_in, const PassParams& p, long long batch,
+                                    float2* work, float2* grad_in, float* grad_phase, float* grad_amp,
+                                    float2* grad_mask, cudaStream_t s);
 
 }  // namespace top
