@@ -825,7 +825,7 @@ top_status transfer_full_table(top_handle h, int Py, int Px, double dy, double d
     c.wsplit = cy.wsplit;
     cudaError_t e = launch_di_samples(a, Py, Px, dy, dx, lam, z, st);
     if (e == cudaSuccess) e = launch_czt_pass(cx.L, r, st);
-    if (e == cudaSuccess) e = launch_transpose_rect(b, a, 1, Py, Px, st);
+    if (e == cudaSuccess) e = launch_transpose(b, a, 1, Py, Px, st);
     if (e == cudaSuccess) e = launch_czt_pass(cy.L, c, st);
     const cudaError_t es = cudaStreamSynchronize(st);
     cudaFree(buf);
@@ -970,7 +970,7 @@ top_status bluestein_fields(top_handle h, const Request& q, const Geometry& geo,
     r.tw = cx.tw;
     r.wsplit = cx.wsplit;
     TOP_TRY(timed(h, KK_ROWS_FWD, st, "Bluestein rows", [&] { return launch_czt_pass(cx.L, r, st); }));
-    TOP_TRY(timed(h, KK_AUX, st, "transpose", [&] { return launch_transpose_rect(w1, w2, n, geo.ny, geo.Px, st); }));
+    TOP_TRY(timed(h, KK_AUX, st, "transpose", [&] { return launch_transpose(w1, w2, n, geo.ny, geo.Px, st); }));
     CztParams c{};
     c.mode = CZT_FILTER;
     c.adjoint = q.adjoint;
@@ -996,7 +996,7 @@ top_status bluestein_fields(top_handle h, const Request& q, const Geometry& geo,
     c.wsplit = cy.wsplit;
     c.h = d_h;
     TOP_TRY(timed(h, KK_COLS, st, "Bluestein columns", [&] { return launch_czt_pass(cy.L, c, st); }));
-    TOP_TRY(timed(h, KK_AUX, st, "transpose", [&] { return launch_transpose_rect(w2, w1, n, geo.Px, geo.ny, st); }));
+    TOP_TRY(timed(h, KK_AUX, st, "transpose", [&] { return launch_transpose(w2, w1, n, geo.Px, geo.ny, st); }));
     CztParams v = r;
     v.mode = CZT_INV;
     v.in = w1;
@@ -2480,7 +2480,7 @@ static top_status coh_two_sided(top_handle h, const top_grid* g, const void* src
   q.epi_kind = EPI_FIELD; q.out = dst;
   TOP_TRY(run_propagation(h, q, st));
   TOP_TRY(timed(h, KK_AUX, st, "transpose", [&] {
-    return launch_transpose(static_cast<const float2*>(dst), static_cast<float2*>(t), g->batch, n, st);
+    return launch_transpose(static_cast<const float2*>(dst), static_cast<float2*>(t), g->batch, n, n, st);
   }));
   q.in = t; q.out = t; q.adjoint = 1 - adjoint_r2;
   return run_propagation(h, q, st);
@@ -2488,7 +2488,8 @@ static top_status coh_two_sided(top_handle h, const top_grid* g, const void* src
 // ... and back to [r1][r2] in dst.
 static top_status coh_untranspose(top_handle h, const top_grid* g, const void* t, void* dst, cudaStream_t st) {
   return timed(h, KK_AUX, st, "transpose", [&] {
-    return launch_transpose(static_cast<const float2*>(t), static_cast<float2*>(dst), g->batch, g->ny * g->nx, st);
+    const int n = g->ny * g->nx;
+    return launch_transpose(static_cast<const float2*>(t), static_cast<float2*>(dst), g->batch, n, n, st);
   });
 }
 

@@ -82,7 +82,7 @@ cudaError_t launch_overlap_partials(const float2* psi, const float2* target, lon
 bool onchip_supported(const PassParams& p);
 cudaError_t launch_onchip(const PassParams& p, cudaStream_t s);
 // out[b][c][r] = in[b][r][c] for a batch of [rows][cols] planes.
-cudaError_t launch_transpose_rect(const float2* in, float2* out, long long batch, int rows, int cols, cudaStream_t s);
+cudaError_t launch_transpose(const float2* in, float2* out, long long batch, int rows, int cols, cudaStream_t s);
 
 }  // namespace top
 
@@ -92,7 +92,6 @@ namespace top {
 // (work: the mask's values, ny nx samples)
 cudaError_t launch_coh_modulate(const float2* in, float2* out, const PassParams& p, long long batch, float2* work,
                                 cudaStream_t s);
-cudaError_t launch_transpose(const float2* in, float2* out, long long batch, int n, cudaStream_t s);
 cudaError_t launch_coh_diag(const float2* gamma, float* inten, long long batch, int n, cudaStream_t s);
 cudaError_t launch_coh_diag_backward(const float* gI, float2* grad, long long batch, int n, cudaStream_t s);
 // The end of the backward, from G' transposed: grad_in = conj(M(r1) conj(M(r2))) G'(r1, r2) (optional) and,
