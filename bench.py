@@ -50,7 +50,7 @@ def measured_peaks():
 
 # The sources the passes of the 1024-point plan are compiled from (their unit and every header it
 # includes): a change anywhere else in the library leaves the profiled kernels as they were.
-KERNEL_SOURCES = ("top_unit_m1024.cu", "top_unit.cuh", "top_dispatch.h", "top_czt.cuh", "top_passes.cuh",
+KERNEL_SOURCES = ("top_unit_m1024.cu", "top_unit.cuh", "top_dispatch.h", "top_czt.cuh", "top_device.h", "top_passes.cuh",
                   "top_engine.cuh", "top_internal.h", "top_launch.h", "../../include/top.h")
 
 

@@ -16,6 +16,7 @@
 // IFFT_M(even) + w^-n IFFT_M(odd), combined through shared memory. Group r of a line is half r.
 #pragma once
 
+#include "top_device.h"
 #include "top_engine.cuh"
 #include "top_internal.h"
 #include "top_launch.h"
@@ -106,11 +107,10 @@ __global__ void __launch_bounds__(CztShape<EN>::THREADS, CztShape<EN>::MINB) k_c
 template <class EN>
 cudaError_t launch_czt(const CztParams& p, cudaStream_t s) {
   using SH = CztShape<EN>;
-  if (SH::SMEM > 48 * 1024) {
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_czt<EN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM);
-    if (attr != cudaSuccess) return attr;
-  }
+  static KernelOnDevices setup;
+  int resident = 0;
+  const cudaError_t ready = setup.ready(k_czt<EN>, SH::THREADS, SH::SMEM, &resident);
+  if (ready != cudaSuccess) return ready;
   dim3 grid((p.nlines + SH::LINES - 1) / SH::LINES, p.nfields);
   TOP_LAUNCH(k_czt<EN>, grid, SH::THREADS, SH::SMEM, s, p);
   return cudaGetLastError();
@@ -258,11 +258,10 @@ __global__ void __launch_bounds__(CztSplitShape<EN>::THREADS, CztSplitShape<EN>:
 template <class EN>
 cudaError_t launch_czt_split(const CztParams& p, cudaStream_t s) {
   using SH = CztSplitShape<EN>;
-  if (SH::SMEM > 48 * 1024) {
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_czt_split<EN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM);
-    if (attr != cudaSuccess) return attr;
-  }
+  static KernelOnDevices setup;
+  int resident = 0;
+  const cudaError_t ready = setup.ready(k_czt_split<EN>, SH::THREADS, SH::SMEM, &resident);
+  if (ready != cudaSuccess) return ready;
   dim3 grid((p.nlines + SH::LINES - 1) / SH::LINES, p.nfields);
   TOP_LAUNCH(k_czt_split<EN>, grid, SH::THREADS, SH::SMEM, s, p);
   return cudaGetLastError();

@@ -17,8 +17,6 @@
 // Bound by the FMA pipe and the shared-memory wavefronts, which 16 warps an SM (128 registers: 32
 // samples a thread) overlap better than the 8 that 64 samples a thread allowed. Results agree with
 // the three passes to rounding, not bit for bit.
-#include <atomic>
-
 #include "top_aux.h"
 #include "top_passes.cuh"
 
@@ -217,22 +215,13 @@ bool onchip_supported(const PassParams& p) {
 }
 
 cudaError_t launch_onchip(const PassParams& p, cudaStream_t s) {
-  // SM count of the current device (the grid is two blocks per SM), looked up, and the kernel's shared
-  // memory allowed, on the first launch per device
-  constexpr int kDevices = 64;
-  static std::atomic<int> known[kDevices];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  int sms = dev < kDevices ? known[dev].load(std::memory_order_acquire) : 0;
-  if (sms == 0) {
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_onchip64, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
-    if (e != cudaSuccess) return e;
-    if (dev < kDevices) known[dev].store(sms, std::memory_order_release);
-  }
-  const int grid = p.nfields < 2 * sms ? p.nfields : 2 * sms;
+  // two blocks fit an SM; the fields are taken in turn
+  static KernelOnDevices setup;
+  int resident = 0;
+  const cudaError_t ready = setup.ready(k_onchip64, kThreads, kSmem, &resident);
+  if (ready != cudaSuccess) return ready;
+  if (resident == 0) resident = 2;  // not known: any number of blocks does
+  const int grid = p.nfields < resident ? p.nfields : resident;
   if (grid <= 0) return cudaSuccess;
   TOP_LAUNCH(k_onchip64, grid, kThreads, kSmem, s, p);
   return cudaGetLastError();

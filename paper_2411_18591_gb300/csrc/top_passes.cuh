@@ -34,6 +34,7 @@
 #include <type_traits>
 #include <utility>
 
+#include "top_device.h"
 #include "top_engine.cuh"
 #include "top_internal.h"
 #include "top_launch.h"
@@ -1276,22 +1277,6 @@ __global__ void __launch_bounds__(RowBlock<EX, COPY ? 2 : row_tiles<EX>()>::THRE
 
 // ----------------------------------------------------------------------------- launchers
 
-template <class K>
-inline cudaError_t set_smem(K kernel, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
-// Blocks of a kernel resident on the whole device at the given block shape (0 if unknown).
-template <class K>
-inline int resident_blocks(K kernel, int threads, size_t smem) {
-  int dev = 0, sms = 0, per_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess)
-    return 0;
-  return sms * per_sm;
-}
-
 // The kernels are compiled for the modulation flag sets of common elements (none, a phase mask, a lens
 // or a phase mask behind an aperture) and for flags read at run time.
 constexpr uint32_t kPhase = TOP_MOD_PHASE;
@@ -1320,9 +1305,10 @@ inline cudaError_t tile_map(const PassParams& p, TileMap* map, bool with_wide) {
 template <class EX, bool X2, uint32_t MF, bool COPY>
 cudaError_t launch_rows_fwd_k(const PassParams& p, cudaStream_t s) {
   using SH = RowBlock<EX, row_tiles<EX>()>;
-  static const cudaError_t attr = set_smem(k_rows_fwd<EX, X2, MF, COPY>, SH::SMEM_X);
-  if (attr != cudaSuccess) return attr;
-  static const int resident = resident_blocks(k_rows_fwd<EX, X2, MF, COPY>, SH::THREADS, SH::SMEM_X);
+  static KernelOnDevices setup;
+  int resident = 0;
+  const cudaError_t ready = setup.ready(k_rows_fwd<EX, X2, MF, COPY>, SH::THREADS, SH::SMEM_X, &resident);
+  if (ready != cudaSuccess) return ready;
   PassParams q = p;
   // bulk prefetches move whole 16-byte units
   q.l2_ahead = p.nx % 2 == 0 && !(p.tune_rows & TOP_TUNE_NO_L2_FWD) ? resident : 0;
@@ -1357,9 +1343,10 @@ cudaError_t launch_rows_fwd_t(const PassParams& p, cudaStream_t s) {
 template <class EY, bool X2, int CI>
 cudaError_t launch_cols_k(const PassParams& p, cudaStream_t s) {
   using SH = ColShape<EY>;
-  static const cudaError_t attr = set_smem(k_cols<EY, X2, CI>, SH::SMEM);
-  if (attr != cudaSuccess) return attr;
-  static const int resident = resident_blocks(k_cols<EY, X2, CI>, SH::THREADS, SH::SMEM);
+  static KernelOnDevices setup;
+  int resident = 0;
+  const cudaError_t ready = setup.ready(k_cols<EY, X2, CI>, SH::THREADS, SH::SMEM, &resident);
+  if (ready != cudaSuccess) return ready;
   PassParams q = p;
   q.l2_ahead = !(p.tune_cols & TOP_TUNE_NO_L2_COLS) ? resident : 0;
   dim3 grid((p.Px + SH::COLS - 1) / SH::COLS, p.nfields);
@@ -1374,9 +1361,10 @@ cudaError_t launch_rows_inv_k(const PassParams& p, cudaStream_t s) {
   const int groups = (q.nfields + q.group - 1) / q.group;
   if constexpr (RowShape<EX>::COPY && KIND != EPI_OVERLAP) {
     using SH = RowBlock<EX, 2>;
-    static const cudaError_t attr = set_smem(k_rows_inv<EX, X2, KIND, MF, true>, SH::SMEM_DUO);
-    if (attr != cudaSuccess) return attr;
-    static const int resident = resident_blocks(k_rows_inv<EX, X2, KIND, MF, true>, SH::THREADS, SH::SMEM_DUO);
+    static KernelOnDevices setup;
+    int resident = 0;
+    const cudaError_t ready = setup.ready(k_rows_inv<EX, X2, KIND, MF, true>, SH::THREADS, SH::SMEM_DUO, &resident);
+    if (ready != cudaSuccess) return ready;
     if (copies_in<EX>(p, resident)) {
       TileMap map{};
       const cudaError_t e = tile_map<EX>(p, &map, true);
@@ -1388,8 +1376,10 @@ cudaError_t launch_rows_inv_k(const PassParams& p, cudaStream_t s) {
     }
   }
   using SH = RowBlock<EX, row_tiles<EX>()>;
-  static const cudaError_t attr = set_smem(k_rows_inv<EX, X2, KIND, MF, false>, SH::SMEM_X);
-  if (attr != cudaSuccess) return attr;
+  static KernelOnDevices setup;
+  int resident = 0;
+  const cudaError_t ready = setup.ready(k_rows_inv<EX, X2, KIND, MF, false>, SH::THREADS, SH::SMEM_X, &resident);
+  if (ready != cudaSuccess) return ready;
   dim3 grid((q.ny + SH::BLOCK_ROWS - 1) / SH::BLOCK_ROWS, groups);
   TOP_LAUNCH((k_rows_inv<EX, X2, KIND, MF, false>), grid, SH::THREADS, SH::SMEM_X, s, q, TileMap{});
   return cudaGetLastError();
@@ -1419,9 +1409,10 @@ template <class EX, bool X2, uint32_t MF>
 cudaError_t launch_rows_chain_k(const PassParams& pa, const PassParams& pb, cudaStream_t s) {
   if constexpr (RowShape<EX>::COPY) {
     using SH = RowBlock<EX, 2>;
-    static const cudaError_t attr = set_smem(k_rows_chain<EX, X2, MF, true>, SH::SMEM_DUO);
-    if (attr != cudaSuccess) return attr;
-    static const int resident = resident_blocks(k_rows_chain<EX, X2, MF, true>, SH::THREADS, SH::SMEM_DUO);
+    static KernelOnDevices setup;
+    int resident = 0;
+    const cudaError_t ready = setup.ready(k_rows_chain<EX, X2, MF, true>, SH::THREADS, SH::SMEM_DUO, &resident);
+    if (ready != cudaSuccess) return ready;
     if (copies_in<EX>(pa, resident)) {
       TileMap map{};
       const cudaError_t e = tile_map<EX>(pa, &map, false);
@@ -1434,8 +1425,10 @@ cudaError_t launch_rows_chain_k(const PassParams& pa, const PassParams& pb, cuda
     }
   }
   using SH = RowBlock<EX, row_tiles<EX>()>;
-  static const cudaError_t attr = set_smem(k_rows_chain<EX, X2, MF, false>, SH::SMEM_X);
-  if (attr != cudaSuccess) return attr;
+  static KernelOnDevices setup;
+  int resident = 0;
+  const cudaError_t ready = setup.ready(k_rows_chain<EX, X2, MF, false>, SH::THREADS, SH::SMEM_X, &resident);
+  if (ready != cudaSuccess) return ready;
   dim3 grid((pa.ny + SH::BLOCK_ROWS - 1) / SH::BLOCK_ROWS, pa.nfields);
   TOP_LAUNCH((k_rows_chain<EX, X2, MF, false>), grid, SH::THREADS, SH::SMEM_X, s, pa, pb, TileMap{});
   return cudaGetLastError();

@@ -1,0 +1,96 @@
+"""What the library's host side asks of the CUDA runtime: its objects linked against a stand-in runtime
+(fake_cudart.cpp) that records launches instead of running them. Needs no GPU and touches none."""
+import ctypes as C
+import glob
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+N = 512
+
+
+class Fake:
+    """The library on the stand-in runtime, called with made-up device addresses."""
+
+    def __init__(self, path, lib):
+        self.dll = C.CDLL(path)
+        for name, (res, args) in lib.SIGNATURES.items():
+            fn = getattr(self.dll, name)
+            fn.restype, fn.argtypes = res, args
+        self.dll.fake_kernel.restype = C.c_char_p
+        self.lib = lib
+        self.buffers = []
+
+    def field(self, samples):
+        """Address of a 16-byte aligned "device" array of complex64 samples (never read or written)."""
+        raw = C.create_string_buffer(8 * samples + 16)
+        self.buffers.append(raw)
+        return (C.addressof(raw) + 15) // 16 * 16
+
+    def handle(self, device=0):
+        h = C.c_void_p()
+        assert self.dll.top_create(C.byref(h), device) == 0
+        return h
+
+    def grid(self, batch, ny, nx, pad=2.0):
+        return C.byref(self.lib.TopGrid(batch, ny, nx, 8e-6, 8e-6, pad, 0, 0))
+
+    def one(self, v):
+        return self.lib.doubles([v])
+
+    def launches(self):
+        return [self.dll.fake_kernel(i).decode() for i in range(self.dll.fake_launches())]
+
+    def error(self):
+        return self.dll.top_last_error().decode()
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    from paper_2411_18591_gb300 import _lib, build
+    build.build()
+    objects = sorted(glob.glob(os.path.join(build.OUT_DIR, "*.o")))
+    if len(objects) != len(glob.glob(os.path.join(build.CSRC, "*.cu"))):
+        build.build(force=True)
+        objects = sorted(glob.glob(os.path.join(build.OUT_DIR, "*.o")))
+    cuda = os.path.join(os.path.dirname(os.path.dirname(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc")), "include")
+    out = str(tmp_path_factory.mktemp("fake") / "libtop_fake.so")
+    # -Bsymbolic: the stand-in's runtime calls also where a real one is loaded in the process
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", build.CSRC, "-I", cuda,
+                    os.path.join(ROOT, "tests", "fake_cudart.cpp"), *objects, "-o", out, "-lpthread"], check=True)
+    return Fake(out, _lib)
+
+
+@pytest.fixture(autouse=True)
+def clean(fake):
+    fake.dll.fake_waits_run_out(0)
+    fake.dll.fake_reset()
+    yield
+
+
+def run_everywhere(fake, h):
+    """Calls whose kernels need more than the 48 KB of shared memory that every launch may have."""
+    x, y = fake.field(1), fake.field(1)
+    lam, z = fake.one(5e-7), fake.one(0.02)
+    stages = (fake.lib.TopStage * 2)()
+    stages[0].z = stages[1].z = 0.02
+    for batch, n in ((64, 256), (64, N), (32, 1024), (1, 4096), (1, 64), (4, 1021)):
+        assert fake.dll.top_propagate(h, fake.grid(batch, n, n), x, y, lam, z, 1, None, None, None) == 0, (n, fake.error())
+        if n not in (64, 1021):
+            st = fake.dll.top_fused_chain(h, fake.grid(batch, n, n), x, y, None, 1, lam, 1, stages, 2, None)
+            assert st == 0, (n, fake.error())
+
+
+def test_kernels_are_set_up_on_every_device(fake):
+    """A second device of the process gets the kernels' shared memory allowed as the first one did."""
+    for device in (0, 1):
+        fake.dll.fake_reset()
+        run_everywhere(fake, fake.handle(device))
+        n = fake.dll.fake_launches()
+        assert n > 20
+        assert not [fake.launches()[i] for i in range(n) if fake.dll.fake_refused(i)]
+        # table kernels aside, everything ran where the handle is
+        assert all(fake.dll.fake_device_of(i) == device for i in range(n))
