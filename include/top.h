@@ -128,6 +128,14 @@ top_status top_create(top_handle* out, int device);
 top_status top_destroy(top_handle h);
 /* Message of the last failing call on this host thread ("" if none). Never NULL. */
 const char* top_last_error(void);
+/* TOP_ERR_TIMEOUT if a bounded wait inside a kernel ran out since this was last reported, else TOP_OK; h NULL:
+ * for top_propagate_noalloc on the current device. Some passes wait for tile copies and work items in flight,
+ * at most about two seconds each; a kernel whose wait runs out drops the rest of its tiles and returns, so the
+ * outputs of its call are not valid. Like every asynchronous error it shows late: the next call on the handle
+ * (or the next no-alloc call on the device) that finds it returns TOP_ERR_TIMEOUT and launches nothing; repeat
+ * it. Ask here after a synchronisation to learn of it without another call, and after replays of a captured
+ * graph, which make none. Does not synchronise; reporting clears it. */
+top_status top_check_waits(top_handle h);
 /* Static name of a status code. */
 const char* top_status_string(top_status s);
 /* TOP_ABI_VERSION of the loaded library. */
@@ -247,7 +255,7 @@ top_status top_fused_chain_backward(top_handle h, const top_grid* g, const void*
  * whose single field and table do not fit is rejected with TOP_ERR_UNSUPPORTED before
  * anything is launched.
  * The first call on a device looks up the scratch address (cudaGetSymbolAddress, which loads
- * that module): make it before any stream capture. Calls share the scratch, so two calls in
+ * that module) and maps one word of host memory: make it before any stream capture. Calls share the scratch, so two calls in
  * flight at once on one device (other streams, other threads) race; order them on one stream or
  * synchronise between them.
  * in, out: complex64 [batch][ny][nx] device, 16-byte aligned (in == out allowed); lambda, z:

@@ -10,6 +10,7 @@ from .binding import (Modulation, Stage, top_fused_chain, top_fused_chain_backwa
                       top_propagate_intensity_backward, top_intensity, top_intensity_backward, top_propagate_noalloc, top_propagate_overlap, top_propagate_ragged, top_overlap_loss, top_resample, top_resample_backward, top_zcritical)
 from .binding import (autotune_clear, autotune_get, autotune_load, autotune_save, autotune_set,  # noqa: F401
                       top_autotune)
+from .binding import check_waits  # noqa: F401
 from .binding import (circular_polarizer, linear_polarizer, top_field_power, top_jones,  # noqa: F401
                       top_jones_backward, waveplate)
 from ._lib import TopError  # noqa: F401

@@ -62,6 +62,7 @@ SIGNATURES = {
     "top_last_error": (C.c_char_p, []),
     "top_status_string": (C.c_char_p, [C.c_int]),
     "top_version": (C.c_int, []),
+    "top_check_waits": (C.c_int, [_P]),
     "top_set_workspace_limit": (C.c_int, [_P, C.c_uint64]),
     "top_plan_query": (C.c_int, [_GRID, C.POINTER(C.c_int64), C.POINTER(C.c_int64), C.POINTER(C.c_uint64)]),
     "top_zcritical": (C.c_double, [C.c_double, C.c_double, C.c_double]),

@@ -659,6 +659,12 @@ def top_zcritical(L: float, dx: float, lam: float) -> float:
     return _lib.load().top_zcritical(L, dx, lam)
 
 
+def check_waits(device=None, noalloc: bool = False) -> None:
+    """Raise TopError if a bounded wait inside a kernel ran out since the last report (after a synchronisation,
+    or after replaying a captured graph). ``noalloc``: of top_propagate_noalloc on the current device."""
+    check(_lib.load().top_check_waits(None if noalloc else handle(device)))
+
+
 def profile_enable(enable: bool = True, device=None) -> None:
     check(_lib.load().top_profile_enable(handle(device), 1 if enable else 0))
 

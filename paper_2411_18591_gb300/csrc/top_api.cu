@@ -111,14 +111,16 @@ struct top_ctx {
 
 namespace {
 
+// TOP_ERR_TIMEOUT once if a kernel's bounded wait has run out since the word was last looked at.
+top_status waits_status(volatile int* fault) {
+  if (!fault || !*fault) return TOP_OK;
+  *fault = 0;
+  return fail(TOP_ERR_TIMEOUT, "a bounded wait of an earlier call's kernel ran out; that call's results are not valid");
+}
+
 top_status bind(top_handle h) {
   TOP_CUDA(cudaSetDevice(h->device), "cudaSetDevice");
-  volatile int* fault = h->fault;
-  if (fault && *fault) {
-    *fault = 0;
-    return fail(TOP_ERR_INTERNAL, "a tile copy of an earlier call did not complete; its results are not valid");
-  }
-  return TOP_OK;
+  return waits_status(h->fault);
 }
 
 template <class T>
@@ -1752,7 +1754,7 @@ top_status run_ragged(top_handle h, int count, const top_grid* grids, const void
 
     PassParams p{};
     set_geometry(p, geo.ny, geo.nx, geo.Py, geo.Px);
-  p.fault = h->fault_dev;
+    p.fault = h->fault_dev;
     p.method = grids[grp[0]].method;
     p.adjoint = backward ? 1 : 0;
     p.src_kind = SRC_FIELD;
@@ -1841,15 +1843,8 @@ top_status top_create(top_handle* out, int device) {
   });
   top_ctx* h = new top_ctx();
   h->device = device;
-  void* word = nullptr;
-  e = cudaHostAlloc(&word, sizeof(int), cudaHostAllocMapped);
-  if (e == cudaSuccess) {
-    h->fault = static_cast<int*>(word);
-    *h->fault = 0;
-    e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->fault_dev), word, 0);
-  }
+  e = fault_word(&h->fault, &h->fault_dev);
   if (e != cudaSuccess) {
-    if (word) cudaFreeHost(word);
     delete h;
     return cuda_fail(e, "cudaHostAlloc(fault word)");
   }
@@ -2673,12 +2668,11 @@ namespace {
 
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
-// Address of the static scratch on the current device (looked up once per device).
-top_status noalloc_scratch(void** out) {
-  const cudaError_t e = noalloc_scratch_address(out);
+top_status noalloc_scratch_status(NoallocScratch* out, bool load) {
+  const cudaError_t e = noalloc_scratch(out, load);
   if (e == cudaErrorInvalidDevice) return fail(TOP_ERR_UNSUPPORTED, "device beyond the ones the static scratch supports");
-  if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(static scratch)");
-  return TOP_OK;
+  if (e != cudaSuccess) return cuda_fail(e, "static scratch");
+  return waits_status(out->fault);
 }
 
 // Append a table to the host image at a 256-byte boundary; returns its byte offset.
@@ -2735,9 +2729,9 @@ top_status propagate_noalloc(const top_grid* g, const void* in, void* out, const
   const int slots = int(std::min<int64_t>({chunk, distinct, int64_t(kMaxSets)}));
   const size_t table_bytes = tw_bytes + size_t(slots) * set_bytes;
 
-  void* scratch = nullptr;
-  TOP_TRY(noalloc_scratch(&scratch));
-  unsigned char* base = static_cast<unsigned char*>(scratch);
+  NoallocScratch scratch;
+  TOP_TRY(noalloc_scratch_status(&scratch, true));
+  unsigned char* base = static_cast<unsigned char*>(scratch.mem);
   float2* ws = reinterpret_cast<float2*>(base + table_bytes);
 
   // twiddles: written in stream order by kernels that carry them in their parameters (no copy from
@@ -2751,6 +2745,7 @@ top_status propagate_noalloc(const top_grid* g, const void* in, void* out, const
 
   PassParams p{};
   set_geometry(p, geo.ny, geo.nx, geo.Py, geo.Px);
+  p.fault = scratch.fault_dev;
   p.method = g->method;
   p.adjoint = 0;
   p.src_kind = SRC_FIELD;
@@ -2818,4 +2813,10 @@ top_status propagate_noalloc(const top_grid* g, const void* in, void* out, const
 extern "C" top_status top_propagate_noalloc(const top_grid* g, const void* in, void* out, const double* lambda,
                                             const double* z, int64_t n_lz, void* stream) {
   return propagate_noalloc(g, in, out, lambda, z, n_lz, static_cast<cudaStream_t>(stream));
+}
+
+extern "C" top_status top_check_waits(top_handle h) {
+  if (h) return waits_status(h->fault);
+  NoallocScratch scratch;
+  return noalloc_scratch_status(&scratch, false);
 }

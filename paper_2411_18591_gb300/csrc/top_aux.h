@@ -16,9 +16,16 @@ constexpr int kMseBlocks = 1024;
 // waits for the stream and cannot be captured in a CUDA graph), no pinned staging to keep alive.
 cudaError_t launch_put(void* dst, const void* src, size_t bytes, cudaStream_t s);
 
-// Device address of the static scratch of top_propagate_noalloc (TOP_NOALLOC_SCRATCH_BYTES) on the
-// current device, looked up with cudaGetSymbolAddress on the first call per device.
-cudaError_t noalloc_scratch_address(void** out);
+// The static scratch of top_propagate_noalloc (TOP_NOALLOC_SCRATCH_BYTES) on the current device and its word
+// for waits that run out; looked up (with `load`; otherwise all NULL until then) once per device.
+struct NoallocScratch {
+  void* mem;
+  int* fault;
+  int* fault_dev;
+};
+cudaError_t noalloc_scratch(NoallocScratch* out, bool load);
+// A host-mapped word (0) and its address on the current device: PassParams::fault of the kernels' launches.
+cudaError_t fault_word(int** host, int** device);
 
 cudaError_t launch_modulate(const PassParams& p, cudaStream_t s);
 cudaError_t launch_modulate_backward(const PassParams& p, cudaStream_t s);

@@ -14,23 +14,42 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[TOP_NOALLOC_SCR
 namespace {
 constexpr int kNoallocDevices = 64;
 std::mutex g_mutex;
-void* g_addr[kNoallocDevices] = {};
+NoallocScratch g_scratch[kNoallocDevices] = {};
 }  // namespace
 
-cudaError_t noalloc_scratch_address(void** out) {
+cudaError_t noalloc_scratch(NoallocScratch* out, bool load) {
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kNoallocDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(g_mutex);
-  if (!g_addr[dev]) {
+  NoallocScratch& s = g_scratch[dev];
+  if (!s.mem && load) {
     void* p = nullptr;
     e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
     if (e != cudaSuccess) return e;
     if (!p) return cudaErrorInvalidSymbol;
-    g_addr[dev] = p;
+    e = fault_word(&s.fault, &s.fault_dev);
+    if (e != cudaSuccess) return e;
+    s.mem = p;
   }
-  *out = g_addr[dev];
+  *out = s;
+  return cudaSuccess;
+}
+
+cudaError_t fault_word(int** host, int** device) {
+  void* word = nullptr;
+  void* mapped = nullptr;
+  cudaError_t e = cudaHostAlloc(&word, sizeof(int), cudaHostAllocMapped);
+  if (e != cudaSuccess) return e;
+  e = cudaHostGetDevicePointer(&mapped, word, 0);
+  if (e != cudaSuccess) {
+    cudaFreeHost(word);
+    return e;
+  }
+  *host = static_cast<int*>(word);
+  **host = 0;
+  *device = static_cast<int*>(mapped);
   return cudaSuccess;
 }
 

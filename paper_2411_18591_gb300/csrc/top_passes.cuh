@@ -331,8 +331,9 @@ struct Tickets {
     int item = -1;
     if (top_mbar_wait(&s->bar, s->parity, kWaitCycles)) {
       item = top_ticket(s->answer);
-    } else if (fault) {
-      *fault = 1;
+    } else {
+      if (fault) *fault = 1;
+      top_mbar_wait(&s->bar, s->parity, kWaitCycles);  // the answer may still come: not into another block's memory
     }
     s->parity ^= 1;
     if (item < 0) {
@@ -456,6 +457,8 @@ struct TileFeed {
       const bool ok = top_mbar_wait(s->full + g, turn, kWaitCycles);
       if (!ok) {
         if (fault) *fault = 1;
+        // what is still in flight lands before the block leaves its memory to another
+        top_mbar_wait(s->full + g, turn, kWaitCycles);
         if (s->tickets.open) top_mbar_wait(&s->tickets.bar, s->tickets.parity, kWaitCycles);
       }
       const int it = s->item[g], ff = s->f[g];

@@ -94,3 +94,30 @@ def test_kernels_are_set_up_on_every_device(fake):
         assert not [fake.launches()[i] for i in range(n) if fake.dll.fake_refused(i)]
         # table kernels aside, everything ran where the handle is
         assert all(fake.dll.fake_device_of(i) == device for i in range(n))
+
+
+def test_waits_that_run_out_are_reported(fake):
+    """By the next call on the handle, or by top_check_waits without one; once; and for the no-alloc call too."""
+    x, y = fake.field(1), fake.field(1)
+    lam, z = fake.one(5e-7), fake.one(0.02)
+    h, other = fake.handle(), fake.handle()
+    call = lambda who: fake.dll.top_propagate(who, fake.grid(64, N, N), x, y, lam, z, 1, None, None, None)
+    noalloc = lambda: fake.dll.top_propagate_noalloc(fake.grid(3, N, N), x, y, lam, z, 1, None)
+    assert call(h) == call(other) == noalloc() == 0
+    assert [fake.dll.top_check_waits(who) for who in (h, other, None)] == [0, 0, 0]
+    fake.dll.fake_waits_run_out(1)
+    assert call(h) == 0 and noalloc() == 0  # asynchronous: the calls themselves do not know
+    fake.dll.fake_waits_run_out(0)
+    assert fake.dll.top_check_waits(other) == 0  # a handle's own
+    timeout = 5
+    for who in (h, None):
+        assert fake.dll.top_check_waits(who) == timeout
+        assert "ran out" in fake.error()
+        assert fake.dll.top_check_waits(who) == 0
+    fake.dll.fake_waits_run_out(1)
+    assert call(h) == 0 and noalloc() == 0
+    fake.dll.fake_waits_run_out(0)
+    fake.dll.fake_reset()
+    assert call(h) == timeout and noalloc() == timeout
+    assert fake.dll.fake_launches() == 0
+    assert call(h) == 0 and noalloc() == 0
