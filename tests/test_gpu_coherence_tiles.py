@@ -59,3 +59,20 @@ def test_coherence_backward_tiles(T, ny, nx, pad, batch):
     out = T.top_propagate_coherence(dev(gamma), d, d, lam, z, pad, mask=mod)
     fwd = [O.propagate_coherence(O.modulate_coherence(x.astype(np.complex128), m), d, d, lam, z, pad) for x in gamma]
     assert rel_l2(out.cpu().numpy(), np.stack(fwd)) < TOL
+
+
+def test_mask_gradient_sums_round_little(T):
+    """The sums over a 64^4 tensor alone, against the same sums in float64 of the call's own grad_in. A term takes
+    eight roundings (its products and the mask's values), the sums at most sixteen levels of rounding: in
+    quadrature sqrt(24) times the rms of one, 2^-24 / sqrt 3."""
+    n, d, lam, z = 64, 10e-6, 633e-9, 0.2
+    g = torch.Generator(device="cuda").manual_seed(4)
+    cplx = lambda: torch.randn((n,) * 4, generator=g, device="cuda", dtype=torch.complex64)
+    gamma, grad = cplx(), cplx()
+    phi = (torch.rand((n, n), generator=g, device="cuda") * 2 - 1) * np.pi
+    gp = torch.zeros_like(phi)
+    gin = T.top_propagate_coherence_backward(grad, d, d, lam, z, mask=T.Modulation(phase=phi), saved_in=gamma, grad_phase=gp)
+    # dL/dphi(r) = sum_s Im(gin(r, s) conj(gamma(r, s))) - sum_s Im(gin(s, r) conj(gamma(s, r)))
+    t = (gin.reshape(n * n, n * n).to(torch.complex128) * gamma.reshape(n * n, n * n).to(torch.complex128).conj()).imag
+    ref = (t.sum(1) - t.sum(0)).reshape(n, n)
+    assert float((gp - ref).norm() / ref.norm()) < np.sqrt(24 / 3) * 2.0 ** -24
