@@ -2457,7 +2457,7 @@ static top_status coh_check(const top_grid* g, const double* lambda, const doubl
 static top_status coh_buffers(top_handle h, const top_grid* g, void** t, float2** work) {
   const size_t n = size_t(g->ny) * g->nx;
   const size_t tensor = (sizeof(float2) * size_t(g->batch) * n * n + 255) / 256 * 256;
-  TOP_TRY(coh_scratch(h, tensor + coh_work(int(n)), t));
+  TOP_TRY(coh_scratch(h, tensor + coh_work(int(n), g->batch), t));
   *work = reinterpret_cast<float2*>(static_cast<char*>(*t) + tensor);
   return TOP_OK;
 }

@@ -790,18 +790,36 @@ __global__ void __launch_bounds__(256) k_coh_diag_backward(const float* gI, floa
 
 // The end of the coherence backward in one pass over its two tensors: G' (transposed, Gt[r2][r1]) back to
 // [r1][r2], times conj(M(r1) conj(M(r2))) into out (if wanted), and, with the saved input Gm, the sums of
-// the mask gradient's row and column terms over the block's kCohRows x kCohCols samples (part_rows
-// [column block][r1], part_cols[row block][r2], each in a fixed order). Bound by HBM: 402 MB on a 64^4
-// tensor (two tensors read, one written), where the transpose, the two sums and the modulation as passes
-// of their own moved 1.2 GB (246 us).
+// the mask gradient's row and column terms over the block's kCohRows x kCohCols samples of `per` tensors of
+// the batch (slice blockIdx.z: part_rows[slice][column block][r1], part_cols[slice][row block][r2], each in a
+// fixed order). Bound by HBM: 402 MB on a 64^4 tensor (two tensors read, one written), where the transpose,
+// the two sums and the modulation as passes of their own moved 1.2 GB (246 us).
 constexpr int kCohRows = 64, kCohCols = 128;
+// Small tensors have few blocks (eight at 16 x 16 samples), so a batch of them is cut into slices until the
+// launch has four an SM: 256 tensors of 16 x 16 in one slice took 6.0 ms a call, in slices 5.1.
+constexpr int kCohBlocks = 4 * 152;
+struct CohSlices {
+  int row_blocks, col_blocks;  // of a tensor
+  int count;                   // slices of the batch
+  long long per;               // tensors of a slice
+};
+static CohSlices coh_slices(int n, long long batch) {
+  CohSlices c;
+  c.row_blocks = (n + kCohRows - 1) / kCohRows;
+  c.col_blocks = (n + kCohCols - 1) / kCohCols;
+  const long long want = std::max(1ll, kCohBlocks / ((long long)c.row_blocks * c.col_blocks));
+  c.per = std::max(1ll, (batch + want - 1) / want);
+  c.count = int((batch + c.per - 1) / c.per);
+  return c;
+}
 __global__ void __launch_bounds__(256) k_coh_backward_end(const float2* Gt, const float2* Gm, const float2* mv, int n,
-                                                          long long batch, float2* out, float2* part_rows,
-                                                          float2* part_cols) {
+                                                          long long batch, long long per, float2* out,
+                                                          float2* part_rows, float2* part_cols) {
   __shared__ float2 tile[32][33];
   __shared__ float2 red[8][32];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int r0 = blockIdx.y * kCohRows, c0 = blockIdx.x * kCohCols;
+  const long long b0 = blockIdx.z * per, b1 = min(b0 + per, batch);
   float2 rows[kCohRows / 8];
 #pragma unroll
   for (int k = 0; k < kCohRows / 8; ++k) rows[k] = make_float2(0.f, 0.f);
@@ -811,7 +829,7 @@ __global__ void __launch_bounds__(256) k_coh_backward_end(const float2* Gt, cons
     const float2 mc = col < n ? __ldg(mv + col) : make_float2(0.f, 0.f);
     float2 cols = make_float2(0.f, 0.f);
 #pragma unroll 1
-    for (long long b = 0; b < batch; ++b) {
+    for (long long b = b0; b < b1; ++b) {
       const long long base = b * n * n;
 #pragma unroll
       for (int rb = 0; rb < kCohRows; rb += 32) {
@@ -846,7 +864,7 @@ __global__ void __launch_bounds__(256) k_coh_backward_end(const float2* Gt, cons
       if (ty == 0 && col < n) {
         float2 t = red[0][tx];
         for (int k = 1; k < 8; ++k) t = c_add(t, red[k][tx]);
-        part_cols[(long long)blockIdx.y * n + col] = t;
+        part_cols[((long long)blockIdx.z * gridDim.y + blockIdx.y) * n + col] = t;
       }
       __syncthreads();
     }
@@ -859,7 +877,7 @@ __global__ void __launch_bounds__(256) k_coh_backward_end(const float2* Gt, cons
       for (int d = 16; d > 0; d >>= 1)
         t = c_add(t, make_float2(__shfl_xor_sync(0xffffffffu, t.x, d), __shfl_xor_sync(0xffffffffu, t.y, d)));
       const int row = r0 + (k / 4) * 32 + ty + 8 * (k % 4);
-      if (tx == 0 && row < n) part_rows[(long long)blockIdx.x * n + row] = t;
+      if (tx == 0 && row < n) part_rows[((long long)blockIdx.z * gridDim.x + blockIdx.x) * n + row] = t;
     }
   }
 }
@@ -903,8 +921,9 @@ __global__ void __launch_bounds__(32 * kCohFinishWarps) k_coh_grad_finish(const 
   }
 }
 
-size_t coh_work(int n) {
-  return sizeof(float2) * size_t(n) * (1 + (n + kCohCols - 1) / kCohCols + (n + kCohRows - 1) / kCohRows);
+size_t coh_work(int n, long long batch) {
+  const CohSlices c = coh_slices(n, batch);
+  return sizeof(float2) * size_t(n) * (1 + size_t(c.count) * size_t(c.row_blocks + c.col_blocks));
 }
 
 cudaError_t launch_coh_modulate(const float2* in, float2* out, const PassParams& p, long long batch, float2* work,
@@ -936,18 +955,20 @@ cudaError_t launch_coh_backward_end(const float2* Gt, const float2* gamma_in, co
                                     float2* work, float2* grad_in, float* grad_phase, float* grad_amp,
                                     float2* grad_mask, cudaStream_t s) {
   const int n = p.ny * p.nx;
-  const dim3 grid((n + kCohCols - 1) / kCohCols, (n + kCohRows - 1) / kCohRows);
+  const CohSlices c = coh_slices(n, batch);
+  const dim3 grid(c.col_blocks, c.row_blocks, c.count);
+  const int nrows = c.count * c.col_blocks, ncols = c.count * c.row_blocks;  // partials a sample
   float2* mv = work;
   float2* rows = work + n;
-  float2* cols = rows + size_t(grid.x) * n;
+  float2* cols = rows + size_t(nrows) * n;
   TOP_LAUNCH(k_coh_mask_values, (n + 255) / 256, 256, 0, s, p, n, mv);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  TOP_LAUNCH(k_coh_backward_end, grid, dim3(32, 8), 0, s, Gt, gamma_in, mv, n, batch, grad_in, rows, cols);
+  TOP_LAUNCH(k_coh_backward_end, grid, dim3(32, 8), 0, s, Gt, gamma_in, mv, n, batch, c.per, grad_in, rows, cols);
   e = cudaGetLastError();
   if (e != cudaSuccess || !gamma_in) return e;
   TOP_LAUNCH(k_coh_grad_finish, (n + kCohFinishWarps - 1) / kCohFinishWarps, 32 * kCohFinishWarps, 0, s, p, n, rows,
-             int(grid.x), cols, int(grid.y), grad_phase, grad_amp, grad_mask);
+             nrows, cols, ncols, grad_phase, grad_amp, grad_mask);
   return cudaGetLastError();
 }
 

@@ -104,8 +104,8 @@ cudaError_t launch_coh_diag_backward(const float* gI, float2* grad, long long ba
 // The end of the backward, from G' transposed: grad_in = conj(M(r1) conj(M(r2))) G'(r1, r2) (optional) and,
 // with the saved input, the mask gradients of
 // g_M(r) = sum_s G(r,s) conj(Gm(r,s)) M(s) + sum_s conj(G(s,r)) Gm(s,r) M(s), summed over the batch in a
-// fixed order. work holds coh_work(ny nx) bytes (the mask's values and the blocks' partial sums).
-size_t coh_work(int n);
+// fixed order. work holds coh_work(ny nx, batch) bytes (the mask's values and the blocks' partial sums).
+size_t coh_work(int n, long long batch);
 cudaError_t launch_coh_backward_end(const float2* Gt, const float2* gamma_in, const PassParams& p, long long batch,
                                     float2* work, float2* grad_in, float* grad_phase, float* grad_amp,
                                     float2* grad_mask, cudaStream_t s);

@@ -76,3 +76,23 @@ def test_mask_gradient_sums_round_little(T):
     t = (gin.reshape(n * n, n * n).to(torch.complex128) * gamma.reshape(n * n, n * n).to(torch.complex128).conj()).imag
     ref = (t.sum(1) - t.sum(0)).reshape(n, n)
     assert float((gp - ref).norm() / ref.norm()) < np.sqrt(24 / 3) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("n,batch", [(16, 160), (16, 3), (32, 9)])
+def test_batches_in_slices(T, n, batch):
+    """A batch that the last pass cuts into slices of several tensors, with a shorter last one: every tensor's
+    grad_in is that of a call of its own, and the mask gradient the sum over the batch (eight roundings a term, up
+    to 24 levels of sums, as above)."""
+    d, lam, z = 10e-6, 633e-9, 0.1
+    g = torch.Generator(device="cuda").manual_seed(n + batch)
+    cplx = lambda: torch.randn((batch,) + (n,) * 4, generator=g, device="cuda", dtype=torch.complex64)
+    gamma, grad = cplx(), cplx()
+    mod = T.Modulation(phase=(torch.rand((n, n), generator=g, device="cuda") * 2 - 1) * np.pi)
+    gp = torch.zeros((n, n), device="cuda")
+    gin = T.top_propagate_coherence_backward(grad, d, d, lam, z, mask=mod, saved_in=gamma, grad_phase=gp)
+    ref = torch.zeros((n, n), dtype=torch.float64, device="cuda")
+    for b in range(batch):
+        assert torch.equal(gin[b], T.top_propagate_coherence_backward(grad[b], d, d, lam, z, mask=mod)), b
+        t = (gin[b].reshape(n * n, n * n).to(torch.complex128) * gamma[b].reshape(n * n, n * n).to(torch.complex128).conj()).imag
+        ref += (t.sum(1) - t.sum(0)).reshape(n, n)
+    assert float((gp - ref).norm() / ref.norm()) < np.sqrt(32 / 3) * 2.0 ** -24

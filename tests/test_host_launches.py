@@ -121,3 +121,26 @@ def test_waits_that_run_out_are_reported(fake):
     assert call(h) == timeout and noalloc() == timeout
     assert fake.dll.fake_launches() == 0
     assert call(h) == 0 and noalloc() == 0
+
+
+def test_coherence_backward_spreads_a_batch_of_small_tensors(fake):
+    """The end of the coherence backward: a batch of small tensors has blocks for the whole chip, a large tensor
+    its own."""
+    h = fake.handle()
+    buf = [fake.field(1) for _ in range(3)]
+    mod = fake.lib.TopMod(flags=fake.lib.TOP_MOD_PHASE, phase=fake.field(1))
+    grads = fake.lib.TopModGrads(saved_in=buf[2], grad_phase=fake.field(1))
+    lam, z = fake.one(5e-7), fake.one(0.02)
+    for batch, n in ((256, 16), (3, 16), (64, 32), (1, 64)):
+        for with_grads in (True, False):
+            fake.dll.fake_reset()
+            st = fake.dll.top_propagate_coherence_backward(h, fake.grid(batch, n, n), buf[0], buf[1], lam, z, C.byref(mod),
+                                                           C.byref(grads) if with_grads else None, None)
+            assert st == 0, fake.error()
+            at = [i for i, k in enumerate(fake.launches()) if "k_coh_backward_end" in k]
+            assert len(at) == 1
+            xyz = (C.c_uint * 3)()
+            fake.dll.fake_grid(at[0], xyz)
+            blocks = xyz[0] * xyz[1]
+            assert blocks == (n * n // 64) * (n * n // 128)
+            assert xyz[2] <= batch and (xyz[2] == batch or blocks * xyz[2] >= 304), (batch, n, list(xyz))
