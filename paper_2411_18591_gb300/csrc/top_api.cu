@@ -1185,9 +1185,13 @@ top_status run_propagation(top_handle h, const Request& q, cudaStream_t st) {
   // per-field parameter sets (the source-side lens tables of this propagation belong to its
   // source modulation, or with upstream stages to the last boundary's)
   const top_mod* src_mod = q.n_up > 0 ? q.up[q.n_up - 1].pre : q.msrc;
-  std::vector<FieldSet> field_sets(B);
-  for (int64_t b = 0; b < B; ++b) {
-    const int64_t i = q.n_lz == 1 ? 0 : b;
+  // one set for the whole batch when it shares lambda and z: with thousands of small fields, a set a field cost
+  // more host time than their kernels take (42 ns a field of 16 x 16 against 14)
+  const bool one_set = q.n_lz == 1;
+  const int64_t nsets = one_set ? 1 : B;
+  auto set_of = [&](int64_t b) { return one_set ? 0 : b; };
+  std::vector<FieldSet> field_sets(nsets);
+  for (int64_t i = 0; i < nsets; ++i) {
     TransferEntry te;
     TOP_TRY(field_transfer(h, g, geo.ny, geo.nx, geo.Py, geo.Px, q.lam[i], q.z[i], st, &te));
     FieldSet fs{};
@@ -1200,18 +1204,17 @@ top_status run_propagation(top_handle h, const Request& q, cudaStream_t st) {
       TOP_TRY(lens_table(h, geo.nx, g->dx, q.lam[i], q.mepi->focal_length, &fs.epi_lx));
       TOP_TRY(lens_table(h, geo.ny, g->dy, q.lam[i], q.mepi->focal_length, &fs.epi_ly));
     }
-    field_sets[b] = fs;
+    field_sets[i] = fs;
   }
   // upstream stages: stage j's transfer table and the lens tables of the boundary modulation its
   // forward row pass applies (none for the first, which starts from the request's source)
-  std::vector<std::vector<FieldSet>> up_sets(size_t(q.n_up), std::vector<FieldSet>(B));
+  std::vector<std::vector<FieldSet>> up_sets(size_t(q.n_up), std::vector<FieldSet>(nsets));
   std::vector<const int2*> up_circ(size_t(q.n_up), nullptr);
   for (int j = 0; j < q.n_up; ++j) {
     const top_mod* bm = j > 0 ? q.up[j - 1].pre : nullptr;
     if (q.up[j].pre && (q.up[j].pre->flags & TOP_MOD_CIRC))
       TOP_TRY(circ_table(h, geo.ny, geo.nx, g->dy, g->dx, q.up[j].pre->radius, &up_circ[j]));
-    for (int64_t b = 0; b < B; ++b) {
-      const int64_t i = q.n_lz == 1 ? 0 : b;
+    for (int64_t i = 0; i < nsets; ++i) {
       TransferEntry te;
       TOP_TRY(field_transfer(h, g, geo.ny, geo.nx, geo.Py, geo.Px, q.lam[i], q.up[j].z, st, &te));
       FieldSet fs{};
@@ -1220,7 +1223,7 @@ top_status run_propagation(top_handle h, const Request& q, cudaStream_t st) {
         TOP_TRY(lens_table(h, geo.nx, g->dx, q.lam[i], bm->focal_length, &fs.src_lx));
         TOP_TRY(lens_table(h, geo.ny, g->dy, q.lam[i], bm->focal_length, &fs.src_ly));
       }
-      up_sets[j][b] = fs;
+      up_sets[j][i] = fs;
     }
   }
   if (q.n_up > 0 && q.msrc == nullptr && src_mod && (src_mod->flags & TOP_MOD_CIRC))
@@ -1335,6 +1338,11 @@ top_status run_propagation(top_handle h, const Request& q, cudaStream_t st) {
     int64_t n = 0;
     p.nsets = 0;
     std::vector<int64_t> rep;
+    if (one_set) {
+      n = std::min<int64_t>(chunk, B - pos);
+      rep.push_back(pos);
+      std::memset(p.set_of, 0, size_t(n));
+    }
     while (pos + n < B && n < chunk) {
       // a whole aligned group of fields at a time
       int64_t gend = std::min<int64_t>(B, pos + n + align);
@@ -1356,7 +1364,7 @@ top_status run_propagation(top_handle h, const Request& q, cudaStream_t st) {
       n = gend - pos;
     }
     p.nsets = int(rep.size());
-    for (size_t k = 0; k < rep.size(); ++k) p.sets[k] = field_sets[rep[k]];
+    for (size_t k = 0; k < rep.size(); ++k) p.sets[k] = field_sets[set_of(rep[k])];
     if (n == 0) return fail(TOP_ERR_UNSUPPORTED, "a group of fields uses more than %d (lambda, z) sets", kMaxSets);
     p.nfields = int(n);
     p.group = int(group);
@@ -1398,7 +1406,7 @@ top_status run_propagation(top_handle h, const Request& q, cudaStream_t st) {
       for (int j = 0; j < q.n_up; ++j) {
         PassParams& u = pu[j];
         u = p;
-        for (size_t k = 0; k < rep.size(); ++k) u.sets[k] = up_sets[j][rep[k]];
+        for (size_t k = 0; k < rep.size(); ++k) u.sets[k] = up_sets[j][set_of(rep[k])];
         u.epi_kind = EPI_FIELD;
         u.out = nullptr;
         u.outf = nullptr;

@@ -144,3 +144,23 @@ def test_coherence_backward_spreads_a_batch_of_small_tensors(fake):
             blocks = xyz[0] * xyz[1]
             assert blocks == (n * n // 64) * (n * n // 128)
             assert xyz[2] <= batch and (xyz[2] == batch or blocks * xyz[2] >= 304), (batch, n, list(xyz))
+
+
+def test_fields_that_share_their_parameters_cost_the_host_once(fake):
+    """8192 fields of one wavelength and distance go out in four launches a pass: with their parameter sets looked
+    up field by field the call took the host some 250 times as long as a single field's."""
+    import time
+    h, x = fake.handle(), fake.field(1)
+    lam, z = fake.one(5e-7), fake.one(0.02)
+
+    def host_time(batch):
+        best = 1e9
+        for _ in range(20):
+            fake.dll.fake_reset()
+            t = time.perf_counter()
+            assert fake.dll.top_propagate(h, fake.grid(batch, 16, 16), x, x, lam, z, 1, None, None, None) == 0
+            best = min(best, time.perf_counter() - t)
+        return best
+
+    host_time(8192)
+    assert host_time(8192) < 50 * host_time(1)
