@@ -905,8 +905,8 @@ top_status bluestein_fields(top_handle h, const Request& q, const Geometry& geo,
   TOP_TRY(czt_plan(h, geo.Px, &cx));
   TOP_TRY(czt_plan(h, geo.Py, &cy));
   std::vector<const float2*> tables(B);
-  for (int64_t b = 0; b < B; ++b) {
-    const double lam = q.lam[q.n_lz == 1 ? 0 : b], z = q.z[q.n_lz == 1 ? 0 : b];
+  for (int64_t b = 0; b < q.n_lz; ++b) {
+    const double lam = q.lam[b], z = q.z[b];
     const int method = resolve_method(g, geo.ny, geo.nx, lam, z);
     if (method == TOP_DI) {
       if (geo.Py < 2 * geo.ny - 1 || geo.Px < 2 * geo.nx - 1)
@@ -916,6 +916,7 @@ top_status bluestein_fields(top_handle h, const Request& q, const Geometry& geo,
     }
     TOP_TRY(transfer_full_table(h, geo.Py, geo.Px, g->dy, g->dx, lam, z, method, st, &tables[b]));
   }
+  if (q.n_lz == 1) std::fill(tables.begin() + 1, tables.end(), tables[0]);
   const long long wplane = (long long)geo.ny * geo.Px;
   const bool pre = q.msrc && q.msrc->flags;
   const bool post = q.mepi && q.mepi->flags;
@@ -947,8 +948,11 @@ top_status bluestein_fields(top_handle h, const Request& q, const Geometry& geo,
       fin = src;
       in_rep = 1;
     }
-    // by kernels that carry the pointers in their parameters: a copy from pageable memory waits for the stream
-    TOP_CUDA(launch_put(d_h, tables.data() + pos, size_t(n) * sizeof(void*), st), "transfer table pointers");
+    const auto chunk_tables = tables.begin() + pos;
+    const bool one_table = q.n_lz == 1 || std::all_of(chunk_tables, chunk_tables + n, [&](const float2* t) { return t == *chunk_tables; });
+    const bool few = one_table || n <= kFewTables;
+    // a longer list by kernels that carry it in their parameters: a copy from pageable memory waits for the stream
+    if (!few) TOP_CUDA(launch_put(d_h, &*chunk_tables, size_t(n) * sizeof(void*), st), "transfer table pointers");
     CztParams r{};
     r.mode = CZT_FWD;
     r.in = fin;
@@ -996,7 +1000,9 @@ top_status bluestein_fields(top_handle h, const Request& q, const Geometry& geo,
     c.bh_inv = cy.bh_inv;
     c.tw = cy.tw;
     c.wsplit = cy.wsplit;
-    c.h = d_h;
+    c.h = few ? nullptr : d_h;
+    c.h_step = one_table ? 0 : 1;
+    if (few) std::copy_n(chunk_tables, one_table ? 1 : n, c.h_few);
     TOP_TRY(timed(h, KK_COLS, st, "Bluestein columns", [&] { return launch_czt_pass(cy.L, c, st); }));
     TOP_TRY(timed(h, KK_AUX, st, "transpose", [&] { return launch_transpose(w2, w1, n, geo.Px, geo.ny, st); }));
     CztParams v = r;

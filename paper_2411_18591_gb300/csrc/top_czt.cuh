@@ -45,6 +45,11 @@ __device__ __forceinline__ void czt_convolve(float2 (&v)[EN::E], float2* buf, in
   EN::inv(v, buf, t, tw);
 }
 
+// The transfer table of field f.
+__device__ __forceinline__ const float2* czt_table(const CztParams& p, int f) {
+  return p.h ? p.h[f] : p.h_few[f * p.h_step];
+}
+
 template <class EN>
 __global__ void __launch_bounds__(CztShape<EN>::THREADS, CztShape<EN>::MINB) k_czt(const __grid_constant__ CztParams p) {
   constexpr int G = EN::G, E = EN::E;
@@ -76,7 +81,7 @@ __global__ void __launch_bounds__(CztShape<EN>::THREADS, CztShape<EN>::MINB) k_c
 
   if (p.mode == CZT_FILTER) {
     // X[k] H[k] conj(c[k]) = conv[k] H[k] / L at k < P (the chirps cancel), zero beyond
-    const float2* hrow = p.h[f] + (long long)li * p.P;
+    const float2* hrow = czt_table(p, f) + (long long)li * p.P;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const int k = EN::in_pos(t, e);
@@ -220,7 +225,7 @@ __global__ void __launch_bounds__(CztSplitShape<EN>::THREADS, CztSplitShape<EN>:
   if (p.mode == CZT_FILTER) {
     // X[k] H[k] conj(c[k]) = conv[k] H[k] / L at k < P (the chirps cancel), zero beyond; times
     // w^k in the odd half
-    const float2* hrow = p.h[f] + (long long)li * p.P;
+    const float2* hrow = czt_table(p, f) + (long long)li * p.P;
 #pragma unroll
     for (int e0 = 0; e0 < E; e0 += CH) {
 #pragma unroll

@@ -164,3 +164,19 @@ def test_fields_that_share_their_parameters_cost_the_host_once(fake):
 
     host_time(8192)
     assert host_time(8192) < 50 * host_time(1)
+
+
+def test_bluestein_calls_write_no_list_of_one_table(fake):
+    """A call at a size without a plan launches its passes alone when its fields share their transfer table, or
+    are few; a longer list of tables is written first."""
+    h, x = fake.handle(), fake.field(1)
+    for batch, sets, writes in ((1, 1, 0), (700, 1, 0), (16, 16, 0), (17, 17, 1)):
+        zs = fake.lib.doubles([0.02 + 0.001 * i for i in range(sets)])
+        lams = fake.lib.doubles([5e-7] * sets)
+        g = fake.grid(batch, 61, 61, 1.0)
+        assert fake.dll.top_propagate(h, g, x, x, lams, zs, sets, None, None, None) == 0, fake.error()  # builds the tables
+        fake.dll.fake_reset()
+        assert fake.dll.top_propagate(h, g, x, x, lams, zs, sets, None, None, None) == 0
+        names = fake.launches()
+        assert len([k for k in names if "k_put" in k]) == writes, (batch, sets, names)
+        assert len(names) == 5 + writes
