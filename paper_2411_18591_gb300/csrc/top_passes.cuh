@@ -1015,6 +1015,7 @@ template <class EX, bool X2, int KIND>
 struct RowEpilogue {
   static constexpr int H = EX::E / 2;
   static constexpr bool REG_ACC = X2 && (KIND == EPI_INTENSITY || KIND == EPI_MODGRAD);
+  static constexpr bool FEW = EX::E < 16;  // samples a thread
   float acc[REG_ACC ? H : 1];
   OvAcc ov;
 
@@ -1044,6 +1045,13 @@ struct RowEpilogue {
       }
     }
   }
+  // a round's partials in memory (read only when they are added to)
+  template <class V, int N, class At>
+  __device__ __forceinline__ static void partials_so_far(const V* part, bool fresh, int nx, At&& of, V (&v)[N]) {
+    if (!part || fresh) return;
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = part[max(0, min(of(k), nx - 1))];
+  }
   // the own slots' samples of row y of field f in group g
   template <uint32_t MF, class Lane>
   __device__ __forceinline__ void field(const PassParams& p, const Lane& c, int f, int g, bool first, int y,
@@ -1061,40 +1069,65 @@ struct RowEpilogue {
     float2* out = KIND == EPI_FIELD ? field_out(p, f) + row0 : (p.out ? p.out + (long long)f * p.out_stride + row0 : nullptr);
     const float2* xs = grads ? p.xs + (long long)f * p.xs_stride + row0 : nullptr;
     const bool fresh = first && !p.part_accumulate;
+    // a kernel compiled for a modulation without an amplitude plane and a mask has no gradients of theirs
+    constexpr bool PHASE_ONLY = MF != TOP_MOD_DYNAMIC && !(MF & (TOP_MOD_AMPLITUDE | TOP_MOD_COMPLEX));
     ov = OvAcc{0.0, 0.0, 0.0};
     // own slots' samples val0
     auto samples = [&](const float2 (&val0)[H], bool hi_part) {
       const OwnSamples<EX, X2> at{c.r(), c.t(), p.ox, hi_part};
       if constexpr (KIND == EPI_MODGRAD) {
-        // val = dL/dy with y = M x (M without conjugation), in two rounds of slots
-        constexpr int N = H % 2 == 0 ? H / 2 : H;
+        // val = dL/dy with y = M x (M without conjugation), in rounds of slots. A round has what it reads in
+        // flight (saved samples, the mask's operands, the partials so far) before it stores anything: loads
+        // do not pass stores, and with a partial loaded, added to and stored slot by slot the pass took 226 us
+        // for eight unpadded fields of 1024 x 1024, now 96. Rounds of four keep the three gradients' operands in
+        // registers at 16 and more samples a thread; fewer samples, and the phase's gradient alone, go in two.
+        constexpr int ROUNDS = PHASE_ONLY || FEW ? (H % 2 == 0 ? 2 : 1) : (H + 3) / 4;
+        constexpr int N = (H + ROUNDS - 1) / ROUNDS;
 #pragma unroll
         for (int k0 = 0; k0 < H; k0 += N) {
+          const auto of = [&](int k) { return k0 + k < H ? at(k0 + k) : -1; };
           float2 mv[N], xv[N];
 #pragma unroll
-          for (int k = 0; k < N; ++k) xv[k] = grads && in_line<X2>(at(k0 + k), nx) ? ldg2(xs + at(k0 + k)) : make_float2(0.f, 0.f);
-          mod_values(m, flags, 0, mr, nx, [&](int k) { return at(k0 + k); }, mv);
+          for (int k = 0; k < N; ++k) xv[k] = grads && k0 + k < H && in_line<X2>(of(k), nx) ? ldg2(xs + of(k)) : make_float2(0.f, 0.f);
+          float so_far[N];
+          if constexpr (!REG_ACC) partials_so_far(p.part_phase ? p.part_phase + part0 : nullptr, fresh, nx, of, so_far);
+          mod_values(m, flags, 0, mr, nx, of, mv);
 #pragma unroll
           for (int k = 0; k < N; ++k) {
-            const int x = at(k0 + k);
-            if (!in_line<X2>(x, nx)) continue;
+            const int x = of(k);
+            if (k0 + k >= H || !in_line<X2>(x, nx)) continue;
             const float2 val = val0[k0 + k];
             if (out) out[x] = c_mulc(val, mv[k]);  // conj(M) dL/dy
             if (p.part_phase) {
               const float2 ys = c_mul(mv[k], xv[k]);
               const float gp = fmaf(val.y, ys.x, -__fmul_rn(val.x, ys.y));  // Im(val conj(y))
               if constexpr (REG_ACC) acc[k0 + k] = __fadd_rn(acc[k0 + k], gp);
-              else p.part_phase[part0 + x] = fresh ? gp : __fadd_rn(p.part_phase[part0 + x], gp);
+              else p.part_phase[part0 + x] = fresh ? gp : __fadd_rn(so_far[k], gp);
             }
-            if (p.part_amp) {
-              // dM/dA = M without its amplitude factor
-              const float2 d = c_mul(mod_at(m, flags & ~TOP_MOD_AMPLITUDE, 0, mr, x), xv[k]);
+          }
+          if (!PHASE_ONLY && p.part_amp) {
+            // dM/dA = M without its amplitude factor
+            float* part = p.part_amp + part0;
+            partials_so_far(part, fresh, nx, of, so_far);
+            mod_values(m, flags & ~TOP_MOD_AMPLITUDE, 0, mr, nx, of, mv);
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+              if (k0 + k >= H || !in_line<X2>(of(k), nx)) continue;
+              const float2 val = val0[k0 + k], d = c_mul(mv[k], xv[k]);
               const float ga = fmaf(val.x, d.x, __fmul_rn(val.y, d.y));  // Re(conj(val) d)
-              p.part_amp[part0 + x] = fresh ? ga : __fadd_rn(p.part_amp[part0 + x], ga);
+              part[of(k)] = fresh ? ga : __fadd_rn(so_far[k], ga);
             }
-            if (p.part_mask) {
-              const float2 gm = c_mulc(val, c_mul(mod_at(m, flags & ~TOP_MOD_COMPLEX, 0, mr, x), xv[k]));  // val conj(M_rest x)
-              p.part_mask[part0 + x] = fresh ? gm : c_add(p.part_mask[part0 + x], gm);
+          }
+          if (!PHASE_ONLY && p.part_mask) {
+            float2* part = p.part_mask + part0;
+            float2 mask_so_far[N];
+            partials_so_far(part, fresh, nx, of, mask_so_far);
+            mod_values(m, flags & ~TOP_MOD_COMPLEX, 0, mr, nx, of, mv);
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+              if (k0 + k >= H || !in_line<X2>(of(k), nx)) continue;
+              const float2 gm = c_mulc(val0[k0 + k], c_mul(mv[k], xv[k]));  // val conj(M_rest x)
+              part[of(k)] = fresh ? gm : c_add(mask_so_far[k], gm);
             }
           }
         }
@@ -1122,16 +1155,38 @@ struct RowEpilogue {
       }
     };
     if (live) {
-      samples(lo, false);
-      if constexpr (!X2) samples(hi, true);
+      if constexpr (X2) {
+        samples(lo, false);
+      } else if constexpr (KIND == EPI_MODGRAD && !FEW) {
+        // one copy of the code for both ends of the line: two spilled 250 bytes and more
+        float2 val[H];
+#pragma unroll 1
+        for (int part = 0; part < 2; ++part) {
+#pragma unroll
+          for (int k = 0; k < H; ++k) val[k] = part ? hi[k] : lo[k];
+          samples(val, part != 0);
+        }
+      } else {
+        samples(lo, false);
+        samples(hi, true);
+      }
     }
   }
 };
 
+// Blocks an SM. The gradients of any set of planes take the next larger number of registers a thread, 128
+// instead of 80 and 80 instead of 64 (64 unpadded fields of 256 x 256: 118 us a backward at 80, 87 at 128).
+template <class SH, int KIND, uint32_t MF>
+constexpr int inv_min_blocks() {
+  constexpr int wider = 65536 / (SH::THREADS * (SH::REGS == 64 ? 80 : 128));
+  return KIND == EPI_MODGRAD && MF == TOP_MOD_DYNAMIC && wider > 0 ? wider : SH::MINB;
+}
+
 // Inverse rows. Without COPY a block holds its tiles for the fields of one group and reads bins straight
 // from the workspace; with it two tiles share a TileFeed.
 template <class EX, bool X2, int KIND, uint32_t MF, bool COPY>
-__global__ void __launch_bounds__(RowBlock<EX, COPY ? 2 : row_tiles<EX>()>::THREADS, RowBlock<EX, COPY ? 2 : row_tiles<EX>()>::MINB)
+__global__ void __launch_bounds__(RowBlock<EX, COPY ? 2 : row_tiles<EX>()>::THREADS,
+                                  inv_min_blocks<RowBlock<EX, COPY ? 2 : row_tiles<EX>()>, KIND, MF>())
     k_rows_inv(const __grid_constant__ PassParams p, const __grid_constant__ TileMap map) {
   constexpr int T = COPY ? 2 : row_tiles<EX>();
   using SH = RowBlock<EX, T>;
@@ -1165,7 +1220,7 @@ __global__ void __launch_bounds__(RowBlock<EX, COPY ? 2 : row_tiles<EX>()>::THRE
 #pragma unroll 1
     for (int f = f0; f < f1; ++f) {
       load_bins<EX>(p, f, c, tile0 + c.qrow(), v);
-      EX::template inv_from<true>(
+      EX::template inv_from<KIND != EPI_MODGRAD || !X2>(
           v, c.qbuf(), c.qt(),
           [&] {
             if (f > f0) c.tile_sync();  // the previous field's trade has been read

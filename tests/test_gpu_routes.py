@@ -1,4 +1,5 @@
-"""Calls whose fields take one of several routes through a kernel, against calls of a field each, bit for bit."""
+"""Calls that take one of several routes through the passes, against calls of a field each (bit for bit) and
+float64 sums, and what a pass may take where a route once held it up."""
 import pytest
 import torch
 
@@ -80,3 +81,63 @@ def test_overlap_sums_do_not_hold_the_pass(T, n, batch):
     x, t = cfield(1, batch, n, n), cfield(2, n, n)
     plain = inverse_rows_us(T, lambda: T.top_propagate(x, d, d, 5e-7, 0.01, 2.0))
     assert inverse_rows_us(T, lambda: T.top_propagate_overlap(x, t, d, d, 5e-7, 0.01, 2.0)) < 5 * plain
+
+
+# padded rows of 512 samples filled, of 512 with both ends of the line folded, of 2000 with odd numbers of rows
+# (lines interleaved in pairs: the last box of a field is clipped), of 1024 filled
+@pytest.mark.parametrize("ny,nx,pad,batch,group", [(512, 512, 1.0, 48, 3), (320, 320, 1.6, 64, 8), (333, 1333, 1.5, 16, 2),
+                                                   (1024, 1024, 1.0, 16, 16)])
+def test_copied_rows_at_other_paddings(T, ny, nx, pad, batch, group):
+    """Row passes that move their tiles by copy, at paddings other than 2: fields, chains, weighted intensities of
+    groups and the gradients of all three planes, against calls of a field each (which do not copy) bit for bit,
+    the sums against float64 sums of theirs (a rounding of 2^-24 each, in quadrature)."""
+    d, z, lam = 6e-6, 0.01, 600e-9
+    g = torch.Generator(device="cuda").manual_seed(ny + nx)
+    x, w = cfield(ny, batch, ny, nx), torch.rand(batch, generator=g, device="cuda") + 0.5
+    planes = dict(phase=torch.rand((ny, nx), generator=g, device="cuda") * 6 - 3,
+                  amplitude=torch.rand((ny, nx), generator=g, device="cuda") + 0.5, mask=cfield(nx, ny, nx))
+    pre = T.Modulation(**planes)
+    stages = [T.Stage(z, pre=pre), T.Stage(0.5 * z, pre=T.Modulation(phase=planes["phase"]))]
+    new = lambda: {"grad_" + k: torch.zeros_like(v) for k, v in planes.items()}
+    one = lambda b: x[b].clone()
+    out = T.top_propagate(x, d, d, lam, z, pad, pre=pre)
+    inten, kept = T.top_propagate_intensity(x, d, d, lam, z, pad, group=group, weights=w, pre=pre, keep_field=True)
+    chain, _ = T.top_fused_chain(x, d, d, lam, stages, pad)
+    grads = new()
+    back = T.top_propagate_backward(x, d, d, lam, z, pad, pre=pre, saved_in=out, **grads)
+    sums = {k: torch.zeros_like(v, dtype=torch.complex128 if v.is_complex() else torch.float64) for k, v in grads.items()}
+    for b in range(batch):
+        o = T.top_propagate(one(b), d, d, lam, z, pad, pre=pre)[0]
+        assert torch.equal(out[b], o) and torch.equal(kept[b], o), b
+        assert torch.equal(chain[b], T.top_fused_chain(one(b), d, d, lam, stages, pad)[0][0]), b
+        g1 = new()
+        assert torch.equal(back[b], T.top_propagate_backward(one(b), d, d, lam, z, pad, pre=pre, saved_in=o.clone(), **g1)), b
+        for k in sums:
+            sums[k] += g1[k]
+    off = lambda a, ref: float((a - ref).norm() / ref.norm())
+    for k in sums:
+        assert off(grads[k], sums[k]) < batch ** 0.5 * 2.0 ** -24, k
+    ref = (w.double()[:, None, None] * kept.to(torch.complex128).abs() ** 2).reshape(-1, group, ny, nx).sum(1)
+    assert off(inten, ref) < (group + 4) ** 0.5 * 2.0 ** -24
+    phase = torch.zeros_like(planes["phase"])
+    only = T.Modulation(phase=planes["phase"])
+    T.top_propagate_backward(x, d, d, lam, z, pad, pre=only, saved_in=out, grad_phase=phase)
+    ref = torch.zeros_like(phase, dtype=torch.float64)
+    for b in range(batch):
+        g1 = torch.zeros_like(phase)
+        T.top_propagate_backward(one(b), d, d, lam, z, pad, pre=only, saved_in=out[b].clone(), grad_phase=g1)
+        ref += g1
+    assert off(phase, ref) < batch ** 0.5 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("n,batch,pad,most", [(1024, 2, 2.0, 1.8), (1024, 8, 1.0, 4.5), (2048, 2, 1.0, 4.5)])
+def test_gradient_epilogue_does_not_hold_the_pass(T, n, batch, pad, most):
+    """The inverse rows with a phase gradient against plain ones: they read the saved field and the partial sums
+    and write these besides (2.2, 6.7 and 6.7 times as long with the partials loaded slot by slot)."""
+    d = 6e-6
+    x, gx = cfield(1, batch, n, n), cfield(2, batch, n, n)
+    gp, phase = torch.zeros((n, n), device="cuda"), torch.rand((n, n), device="cuda")
+    plain = inverse_rows_us(T, lambda: T.top_propagate(x, d, d, 5e-7, 0.01, pad))
+    back = inverse_rows_us(T, lambda: T.top_propagate_backward(gx, d, d, 5e-7, 0.01, pad, pre=T.Modulation(phase=phase),
+                                                               saved_in=x, grad_phase=gp))
+    assert back < most * plain
