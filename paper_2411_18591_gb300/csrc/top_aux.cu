@@ -89,9 +89,10 @@ __global__ void __launch_bounds__(256) k_reduce_partials(const float* part_phase
 }
 
 // MSE: each of kMseBlocks blocks sums a fixed strided subset in float64 (fixed tree order),
-// then one block sums the partials in a fixed order. Bound by bytes in flight: four elements are loaded before
-// any is used (the gradient's stores kept the compiler from moving a later element's loads above them:
-// 16 intensities of 512^2 took 41 us against 37, both kernels).
+// then one block sums the partials in a fixed order. Four elements are loaded before any is used (the
+// gradient's stores kept the compiler from moving a later element's loads above them: 16 intensities of
+// 512^2 took 41 us against 37, both kernels; the 50 MB take 7.4 at the copy rate, so the loads are not
+// what holds them most).
 constexpr int kMseLoads = 4;
 __global__ void __launch_bounds__(256) k_mse_partial(long long n, const float* I, const float* T, float* grad,
                                                      double* partial) {

@@ -357,10 +357,6 @@ struct Engine : Radices<R0, R1, R2, R3> {
     for (int s = 0; s < NS - 1; ++s) b += ((m / weight(s)) % radix(s)) * (span(s) / RL);
     return b;
   }
-  __device__ __forceinline__ static int bin(int t, int e) {
-    const int q = e / RL, j = e - (e / RL) * RL;
-    return kbase(t + G * q) + j * (M / RL);
-  }
 
   template <int S, int DIR>
   __device__ __forceinline__ static void stage(float2 (&v)[E], int t, const float2* __restrict__ tw) {

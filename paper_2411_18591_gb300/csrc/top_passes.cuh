@@ -326,7 +326,7 @@ struct Tickets {
     top_ask_ticket(s->answer, &s->bar);
   }
   // The asked item, or -1; asks for the next one. One thread at a time, in an order that barriers give.
-  __device__ __forceinline__ int take(int* fault, bool again = true) const {
+  __device__ __forceinline__ int take(int* fault) const {
     if (!s->open) return -1;
     int item = -1;
     if (top_mbar_wait(&s->bar, s->parity, kWaitCycles)) {
@@ -338,7 +338,7 @@ struct Tickets {
     s->parity ^= 1;
     if (item < 0) {
       s->open = 0;
-    } else if (again) {
+    } else {
       top_async_fence();  // the answer has been read
       ask();
     }
@@ -887,10 +887,10 @@ __device__ __forceinline__ int line_abs_kx(const PassParams& p, int line) {
 }
 
 // One column per two thread groups, straight between registers and the workspace: the two groups
-// share nothing but the trade before the store, so a block has no barrier of its own. Bound by the L1
-// data path (70 % of its wavefronts: the exchanges, the column's two reads, the H row) and the FMA pipe
-// (55-60 %). Against blocks that staged four-line columns through shared memory: 1024 points 15.7 ->
-// 14.7 us a field, 4096 points 483 -> 379, 1000 points 38 -> 26.
+// share nothing but the trade before the store, so a block has no barrier of its own. Bound by the FMA
+// pipe and the L1 data path together (60 and 62 % of their peaks at 1024 points: the exchanges, the
+// column's two reads, the H row). Against blocks that staged four-line columns through shared memory: 1024
+// points 15.7 -> 12.7 us a field, 4096 points 483 -> 373, 1000 points 38 -> 23.8.
 template <class EY, bool X2, int CI>
 __global__ void __launch_bounds__(ColShape<EY>::THREADS, ColShape<EY>::MINB) k_cols(const __grid_constant__ PassParams p) {
   using SH = ColShape<EY>;
