@@ -204,8 +204,8 @@ typedef struct top_stage {
  * given) and, when `intensity` is non-NULL, |x_K|^2 summed over each `group` consecutive fields
  * (Eq. 14) to intensity [batch / group][ny][nx] (float32). g->input_repeat as in top_propagate.
  * lambda: host, n_lz values (1 or batch), shared by every stage. Results equal the same
- * sequence of top_propagate calls; a boundary whose modulation planes would not fit in shared
- * memory runs as two launches (through `keep`, or a field-sized scratch in the workspace). */
+ * sequence of top_propagate calls; at padded sizes without a plan the stages run as those calls, through
+ * a field-sized scratch. */
 top_status top_fused_chain(top_handle h, const top_grid* g, const void* in, void* out, float* intensity,
                            int64_t group, const double* lambda, int64_t n_lz, const top_stage* stages,
                            int nstages, void* stream);
@@ -220,8 +220,8 @@ top_status top_fused_chain(top_handle h, const top_grid* g, const void* in, void
  * g_0; first_grads (may be NULL) the gradients of stages[0].pre's phase / amplitude / mask from
  * h_1 and its saved_in = x_0, as top_propagate_backward gives them. Each stage boundary (inverse
  * rows of one adjoint propagation, conj(pre) of its element, forward rows of the next) is one
- * fused row pass; padded sizes without a plan, or boundaries whose operands do not fit, run as
- * separate propagations through a field-sized scratch with the same results. Results equal the
+ * fused row pass; padded sizes without a plan run as separate propagations through a field-sized
+ * scratch with the same results. Results equal the
  * sequence top_propagate_intensity_backward (stage K, post NULL) then top_propagate_backward
  * (stage k with post = pre_{k+1}) down to stage 1. lambda: host, n_lz values (1 or batch);
  * g->input_repeat 0 or 1. */
@@ -435,8 +435,8 @@ top_status top_coherence_intensity_backward(top_handle h, const top_grid* g, con
 
 /* Measure the pass variants on g's geometry (padded sizes with a plan of their own; g->batch
  * fields of scratch, allocated and freed by the call -- 16 or more fields at 1024^2 give passes
- * long enough to time) with CUDA events, keep for every pass kind the fastest, and record the
- * choices in the process-wide table for Px/2 (row bits) and Py/2 (column bit). Synchronises the
+ * long enough to time) with CUDA events, keep the faster variant of the forward rows and of the
+ * column pass (with their L2 prefetch or without), and record the choices in the process-wide table for Px/2 (row bits) and Py/2 (column bit). Synchronises the
  * device. rows_flags / cols_flags (may be NULL) receive the entries written. */
 top_status top_autotune(top_handle h, const top_grid* g, uint32_t* rows_flags, uint32_t* cols_flags);
 /* The process-wide table, host-only: set, get (0 when absent), clear. Invalid flags:
@@ -461,8 +461,9 @@ top_status top_profile_enable(top_handle h, int enable);
  * kinds (up to `cap` entries) get static names, ms the summed milliseconds and count the
  * launches since the last call; *n receives the number of kinds written. The kinds are
  * "rows_fwd" (forward row passes), "cols" (column passes), "rows_inv" (inverse row passes),
- * "aux" (losses, reductions, modulations and the other auxiliary kernels) and "rows_chain"
- * (the fused inverse-and-forward row passes between the stages of a system chain). */
+ * "aux" (losses, reductions, modulations and the other auxiliary kernels), "rows_chain"
+ * (the fused inverse-and-forward row passes between the stages of a system chain) and "onchip"
+ * (whole propagations of 64 x 64 fields in one kernel). */
 top_status top_profile_read(top_handle h, int cap, const char** kinds, double* ms, int64_t* count, int* n);
 
 #ifdef __cplusplus

@@ -1249,9 +1249,10 @@ top_status run_propagation(top_handle h, const Request& q, cudaStream_t st) {
   int64_t group = 1;
   if (q.epi_kind == EPI_INTENSITY) group = q.group;
   const bool partials = want_pgrads && shared_mask;
-  const int rows_per_cta_guess = 8;
   if (partials) {
-    const int64_t tiles = (geo.ny + rows_per_cta_guess - 1) / rows_per_cta_guess;
+    // groups enough for four blocks of eight rows an SM (the row tiles have two or four rows, so there are
+    // more); the groups set the order of the sums
+    const int64_t tiles = (geo.ny + 7) / 8;
     const int64_t want_groups = std::max<int64_t>(1, (4 * 152 + tiles - 1) / tiles);
     group = std::max<int64_t>(1, (B + want_groups - 1) / want_groups);
   }
@@ -1906,14 +1907,10 @@ top_status top_autotune(top_handle h, const top_grid* g, uint32_t* rows_flags, u
     tune_set(Mx, (tune_flags(Mx) & ~row_bits) | rows);
     tune_set(My, (tune_flags(My) & ~col_bits) | cols);
   };
-  top_mod lens{};
-  lens.flags = TOP_MOD_LENS;
-  lens.focal_length = 0.1;
   const double lam = 532e-9, z = 0.01;
-  const top_stage stages[2] = {{z, nullptr, nullptr}, {z, &lens, nullptr}};
   top_grid gg = *g;
   gg.input_repeat = 0;
-  // one candidate: a propagation and a two-stage chain, the mean milliseconds per kind over 3 runs
+  // one candidate: a propagation and an intensity's backward, the mean milliseconds per kind over 3 runs
   auto measure = [&](uint32_t rows, uint32_t cols, double (&t)[KK_COUNT]) -> top_status {
     apply(rows, cols);
     for (int rep = 0; rep < 4; ++rep) {
@@ -1927,7 +1924,6 @@ top_status top_autotune(top_handle h, const top_grid* g, uint32_t* rows_flags, u
       b.g = &gg; b.lam = &lam; b.z = &z; b.n_lz = 1; b.adjoint = 1; b.src_kind = SRC_INTENSITY; b.psi_src = x;
       b.gI = static_cast<const float*>(gi); b.group = 1; b.epi_kind = EPI_FIELD; b.out = y;
       TOP_TRY(run_propagation(h, b, nullptr));
-      TOP_TRY(run_chain(h, &gg, x, y, nullptr, 1, &lam, 1, stages, 2, nullptr));
     }
     h->prof = false;
     TOP_CUDA(cudaDeviceSynchronize(), "cudaDeviceSynchronize(autotune)");
