@@ -29,7 +29,11 @@ cudaError_t noalloc_scratch(NoallocScratch* out, bool load) {
     e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
     if (e != cudaSuccess) return e;
     if (!p) return cudaErrorInvalidSymbol;
+    // host memory is mapped here once, also when the thread is capturing a stream
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     e = fault_word(&s.fault, &s.fault_dev);
+    cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) return e;
     s.mem = p;
   }

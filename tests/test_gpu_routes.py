@@ -141,3 +141,29 @@ def test_gradient_epilogue_does_not_hold_the_pass(T, n, batch, pad, most):
     back = inverse_rows_us(T, lambda: T.top_propagate_backward(gx, d, d, 5e-7, 0.01, pad, pre=T.Modulation(phase=phase),
                                                                saved_in=x, grad_phase=gp))
     assert back < most * plain
+
+
+def test_first_noalloc_call_of_a_process_may_be_captured(T):
+    """The look-up of the static scratch and the word beside it does not break a capture under way."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    code = """
+import torch
+import paper_2411_18591_gb300 as T
+x = torch.randn(3, 512, 512, device="cuda", dtype=torch.complex64)
+y, ref = torch.zeros_like(x), torch.zeros_like(x)
+torch.cuda.synchronize()
+graph = torch.cuda.CUDAGraph()
+with torch.cuda.graph(graph):
+    T.top_propagate_noalloc(x, 8e-6, 8e-6, 5e-7, 0.02, out=y)
+graph.replay()
+T.top_propagate_noalloc(x, 8e-6, 8e-6, 5e-7, 0.02, out=ref)
+torch.cuda.synchronize()
+T.check_waits()
+T.check_waits(noalloc=True)
+assert torch.equal(y, ref) and float(y.abs().sum()) > 0
+"""
+    run = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0, run.stderr[-2000:]
