@@ -1143,7 +1143,8 @@ struct RowEpilogue {
           if constexpr (KIND == EPI_INTENSITY) {
             const float i = fmaf(val.x, val.x, __fmul_rn(val.y, val.y));
             if constexpr (REG_ACC) {
-              // the weight and the sum in one rounding for the 32 x 32 plan, in two for the others
+              // the weight and the sum in one rounding for the 32 x 32 plan, in two for the others: results
+              // of either keep the bits they have always had
               acc[k] = EX::NS == 2 && EX::G == 32 ? fmaf(w, i, acc[k]) : __fadd_rn(acc[k], __fmul_rn(w, i));
             } else {
               float* dst = p.outf + (long long)g * p.outf_stride + row0 + x;
