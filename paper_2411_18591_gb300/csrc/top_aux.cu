@@ -247,32 +247,34 @@ __global__ void __launch_bounds__(256) k_transfer_full(float2* h, int Py, int Px
 }
 
 // out[b][c][r] = in[b][r][c] for [rows][cols] planes, through a padded shared tile. Bound by HBM: a thread's
-// sixteen loads are in flight before the first is stored, and rows are read and written 512 bytes at a time
-// (37 us on a 64^4 tensor, 268 MB moved; with four loads a thread and 256 bytes the auxiliary passes of the
-// coherence step took 423 us against 387, those of a 1021^2 forward and backward 193 against 156).
-constexpr int kTile = 64;
+// loads (sixteen for tiles of 64) are in flight before the first is stored, and rows are read and written 512
+// bytes at a time (37 us on a 64^4 tensor, 268 MB moved; in tiles of 32, four loads a thread, the auxiliary
+// passes of the coherence step took 423 us against 387, those of a 1021^2 forward and backward 193 against 156).
+// Planes of at most 32 a side leave three quarters of such a tile empty and keep tiles of 32 (two transposes
+// of 2048 planes of 16 x 16: 13.9 us, in tiles of 64 20.5).
+template <int TILE>
 __global__ void __launch_bounds__(256) k_transpose(const float2* in, float2* out, int rows, int cols) {
-  __shared__ float2 tile[kTile][kTile + 1];
+  __shared__ float2 tile[TILE][TILE + 1];
   const long long base = (long long)blockIdx.z * rows * cols;
-  const int bc = blockIdx.x * kTile, br = blockIdx.y * kTile;
+  const int bc = blockIdx.x * TILE, br = blockIdx.y * TILE;
   const int tx = threadIdx.x, ty = threadIdx.y;
-  float2 v[kTile / 8][2];
+  float2 v[TILE / 8][TILE / 32];
 #pragma unroll
-  for (int j = 0; j < kTile / 8; ++j)
+  for (int j = 0; j < TILE / 8; ++j)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < TILE / 32; ++h) {
       const int r = br + ty + 8 * j, c = bc + tx + 32 * h;
       if (r < rows && c < cols) v[j][h] = in[base + (long long)r * cols + c];
     }
 #pragma unroll
-  for (int j = 0; j < kTile / 8; ++j)
+  for (int j = 0; j < TILE / 8; ++j)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) tile[ty + 8 * j][tx + 32 * h] = v[j][h];
+    for (int h = 0; h < TILE / 32; ++h) tile[ty + 8 * j][tx + 32 * h] = v[j][h];
   __syncthreads();
 #pragma unroll
-  for (int j = 0; j < kTile / 8; ++j)
+  for (int j = 0; j < TILE / 8; ++j)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < TILE / 32; ++h) {
       const int c = bc + ty + 8 * j, r = br + tx + 32 * h;
       if (r < rows && c < cols) out[base + (long long)c * rows + r] = tile[tx + 32 * h][ty + 8 * j];
     }
@@ -731,14 +733,19 @@ cudaError_t launch_transfer_full(float2* h, int Py, int Px, double dy, double dx
   return cudaGetLastError();
 }
 
-cudaError_t launch_transpose(const float2* in, float2* out, long long batch, int rows, int cols, cudaStream_t s) {
+template <int TILE>
+static cudaError_t launch_transpose_tiles(const float2* in, float2* out, long long batch, int rows, int cols, cudaStream_t s) {
   for (long long b0 = 0; b0 < batch; b0 += 65535) {
     const unsigned nb = unsigned(std::min<long long>(65535, batch - b0));
-    dim3 grid((cols + kTile - 1) / kTile, (rows + kTile - 1) / kTile, nb);
+    dim3 grid((cols + TILE - 1) / TILE, (rows + TILE - 1) / TILE, nb);
     const long long off = b0 * rows * cols;
-    TOP_LAUNCH(k_transpose, grid, dim3(32, 8), 0, s, in + off, out + off, rows, cols);
+    TOP_LAUNCH(k_transpose<TILE>, grid, dim3(32, 8), 0, s, in + off, out + off, rows, cols);
   }
   return cudaGetLastError();
+}
+cudaError_t launch_transpose(const float2* in, float2* out, long long batch, int rows, int cols, cudaStream_t s) {
+  return std::max(rows, cols) <= 32 ? launch_transpose_tiles<32>(in, out, batch, rows, cols, s)
+                                    : launch_transpose_tiles<64>(in, out, batch, rows, cols, s);
 }
 
 cudaError_t launch_mse(long long n, const float* I, const float* T, float* grad, double* partial, double* loss,

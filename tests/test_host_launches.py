@@ -180,3 +180,14 @@ def test_bluestein_calls_write_no_list_of_one_table(fake):
         names = fake.launches()
         assert len([k for k in names if "k_put" in k]) == writes, (batch, sets, names)
         assert len(names) == 5 + writes
+
+
+def test_transposes_of_small_planes_fill_their_tiles(fake):
+    """Planes of at most 32 samples a side are transposed in tiles of 32, larger ones in tiles of 64."""
+    h, x = fake.handle(), fake.field(1)
+    lam, z = fake.one(5e-7), fake.one(0.02)
+    for n, tile in ((17, 32), (31, 32), (33, 64), (61, 64)):
+        fake.dll.fake_reset()
+        assert fake.dll.top_propagate(h, fake.grid(64, n, n, 1.0), x, x, lam, z, 1, None, None, None) == 0, fake.error()
+        names = [k for k in fake.launches() if "k_transpose" in k]
+        assert len(names) == 2 and all("k_transpose<%d>" % tile in k for k in names), (n, names)
